@@ -13,7 +13,6 @@
 
 namespace ntc {
 
-constexpr int kTile = 128;       // queries per CTA tile (one per thread)
 constexpr int kHidden = NTC_HIDDEN;
 constexpr int kMaxC = NTC_MAX_CHANNELS;
 constexpr int kMaxGridCh = 20;   // features per cell of one grid (Sec. 6: profile 0.5's G1)
@@ -185,6 +184,16 @@ __device__ __forceinline__ uint32_t cell_index(const Cell& c, int ch, int bits) 
   return (uint32_t)(w >> (bit & 63)) & ((1u << bits) - 1u);
 }
 
+// Level value of quantisation index k: (k - off) q, with k - off formed in
+// the mantissa of 2^23 + k (exact; an integer conversion runs at a quarter of
+// the FP32 rate).
+__device__ __forceinline__ float level_value(uint32_t k, float off23, float q) {
+  return (__uint_as_float(0x4B000000u | k) - off23) * q;
+}
+__device__ __forceinline__ float level_offset(int bits) {
+  return 8388608.f + (float)((1 << (bits - 1)) - 1);
+}
+
 __host__ __device__ __forceinline__ int cell_bytes(int c, int bits) {
   int need = (c * bits + 7) / 8, b = 1;
   while (b < need) b <<= 1;
@@ -222,6 +231,8 @@ __device__ __forceinline__ void vq_cell(const ntc_material& M, int j, int cell,
   }
 }
 
+// F32: the grids are NTC_GRID_F32 and not vector-quantised (the trainers).
+template <bool F32 = false>
 __device__ __forceinline__ void sample_grid(const ntc_material& M, int j, int k, int x, int y,
                                             int wm, int hm, bool noise, uint64_t nkey,
                                             GridSample& gs, Taps* taps_out = nullptr) {
@@ -233,7 +244,7 @@ __device__ __forceinline__ void sample_grid(const ntc_material& M, int j, int k,
   if (taps_out) *taps_out = t;
 #pragma unroll
   for (int ch = 0; ch < kGridPad; ++ch) gs.acc[ch] = 0.f;
-  if (k == 0 && M.vq_books > 0) {
+  if (!F32 && k == 0 && M.vq_books > 0) {
 #pragma unroll
     for (int tp = 0; tp < 4; ++tp) {
       float v[kMaxGridCh];
@@ -244,21 +255,24 @@ __device__ __forceinline__ void sample_grid(const ntc_material& M, int j, int k,
     }
     return;
   }
-  if (M.encoding == NTC_GRID_PACKED) {
+  if (!F32 && M.encoding == NTC_GRID_PACKED) {
     const int bits = k ? M.bits1 : M.bits0;
-    const int off = (1 << (bits - 1)) - 1;
+    const float off = level_offset(bits);
     const int cb = cell_bytes(c, bits);
     const uint8_t* base = static_cast<const uint8_t*>(k ? L.grid1 : L.grid0);
+    Cell cl[4];
 #pragma unroll
-    for (int tp = 0; tp < 4; ++tp) {
-      const Cell cl = load_cell(base, t.cell[tp], cb);
+    for (int tp = 0; tp < 4; ++tp) cl[tp] = load_cell(base, t.cell[tp], cb);
 #pragma unroll
-      for (int ch = 0; ch < kMaxGridCh; ++ch)
-        if (ch < c) {
-          const float v = (float)((int)cell_index(cl, ch, bits) - off) * q;
-          gs.acc[ch] = fmaf(t.w[tp], v, gs.acc[ch]);
-        }
-    }
+    for (int c4 = 0; c4 < kMaxGridCh / 4; ++c4)
+      if (4 * c4 < c) {
+#pragma unroll
+        for (int tp = 0; tp < 4; ++tp)
+#pragma unroll
+          for (int ch = 4 * c4; ch < 4 * c4 + 4; ++ch)
+            if (ch < c)
+              gs.acc[ch] = fmaf(t.w[tp], level_value(cell_index(cl[tp], ch, bits), off, q), gs.acc[ch]);
+      }
   } else {
     const float* base = static_cast<const float*>(k ? L.grid1 : L.grid0);
 #pragma unroll
@@ -292,10 +306,11 @@ __device__ __forceinline__ void sample_grid(const ntc_material& M, int j, int k,
 
 // One latent value of grid k at a cell: dequantised index (packed) or the
 // FP32 value plus this step's noise.
+template <bool F32 = false>
 __device__ __forceinline__ float grid_value(const ntc_material& M, int j, int k, int cell, int ch,
                                             bool noise, uint64_t nkey) {
   const ntc_level& L = M.lv[j];
-  if (k == 0 && M.vq_books > 0) {
+  if (!F32 && k == 0 && M.vq_books > 0) {
     const uint8_t* ib = static_cast<const uint8_t*>(L.grid0) + (size_t)cell * M.vq_books;
     float v = 0.f;
     for (int b = 0; b < M.vq_books; ++b)
@@ -304,7 +319,7 @@ __device__ __forceinline__ float grid_value(const ntc_material& M, int j, int k,
   }
   const int c = k ? M.c1 : M.c0;
   const float q = k ? M.q1 : M.q0;
-  if (M.encoding == NTC_GRID_PACKED) {
+  if (!F32 && M.encoding == NTC_GRID_PACKED) {
     const int bits = k ? M.bits1 : M.bits0;
     const Cell cl = load_cell(static_cast<const uint8_t*>(k ? L.grid1 : L.grid0), cell,
                               cell_bytes(c, bits));
@@ -315,38 +330,62 @@ __device__ __forceinline__ float grid_value(const ntc_material& M, int j, int k,
   return val;
 }
 
+// The features of grid k at texel (x, y) of mip m, through sink(index, value):
+// slots 0 .. (G0: c0 bilinear values, or with learned interpolation, Sec.
+// 4.3.1, the four taps' values concatenated), then G1's c1 bilinear values.
+template <class Sink>
+__device__ __forceinline__ void grid_features(const ntc_material& M, int k, int x, int y, int m,
+                                              bool noise, uint64_t nkey, Sink& sink) {
+  const int j = level_of_mip(m, M.levels);
+  const int wm = mip_dim(M.width, m), hm = mip_dim(M.height, m);
+  const bool learned = M.interp0 == NTC_INTERP_LEARNED;
+  if (k == 0 && learned) {
+    const ntc_level& L = M.lv[j];
+    const Taps t = bilinear_taps(x, y, wm, hm, L.g0_w, L.g0_h);
+    if (M.vq_books == 0 && M.encoding == NTC_GRID_PACKED) {
+      const int cb = cell_bytes(M.c0, M.bits0);
+      const float off = level_offset(M.bits0);
+      Cell cl[4];
+#pragma unroll
+      for (int tp = 0; tp < 4; ++tp) cl[tp] = load_cell(static_cast<const uint8_t*>(L.grid0), t.cell[tp], cb);
+#pragma unroll
+      for (int tp = 0; tp < 4; ++tp)
+        for (int ch = 0; ch < M.c0; ++ch)
+          sink(tp * M.c0 + ch, level_value(cell_index(cl[tp], ch, M.bits0), off, M.q0));
+    } else {
+#pragma unroll 1
+      for (int tp = 0; tp < 4; ++tp)
+        for (int ch = 0; ch < M.c0; ++ch)
+          sink(tp * M.c0 + ch, grid_value(M, j, 0, t.cell[tp], ch, noise, nkey));
+    }
+    return;
+  }
+  GridSample gs;
+  sample_grid(M, j, k, x, y, wm, hm, noise, nkey, gs);
+  const int c = k ? M.c1 : M.c0, s0 = k ? (learned ? 4 * M.c0 : M.c0) : 0;
+#pragma unroll
+  for (int ch = 0; ch < kMaxGridCh; ++ch)
+    if (ch < c) sink(s0 + ch, gs.acc[ch]);
+}
+
+// The slots after the grids: 12 positional-encoding values, m/(M-1), zeros.
+template <class Sink>
+__device__ __forceinline__ void tail_features(const ntc_material& M, int x, int y, int m, Sink& sink) {
+  const int pe = (M.interp0 == NTC_INTERP_LEARNED ? 4 * M.c0 : M.c0) + M.c1;
+  positional_encoding(x, y, pe, sink);
+  sink(pe + 12, M.mips > 1 ? (float)m / (float)(M.mips - 1) : 0.f);
+  for (int i = pe + 13; i < M.k_in; ++i) sink(i, 0.f);
+}
+
 // The MLP input row of texel (x, y, m) (Sec. 4.3, 4.4):
 // [G0 features | G1 features | 12 PE values | m/(M-1) | 0 ...], written
 // through sink(index, value) for indices 0 .. k_in-1.
 template <class Sink>
 __device__ __forceinline__ void featurize(const ntc_material& M, int x, int y, int m, bool noise,
                                           uint64_t nkey, Sink& sink) {
-  const int j = level_of_mip(m, M.levels);
-  const int wm = mip_dim(M.width, m), hm = mip_dim(M.height, m);
-  GridSample gs;
-  int w0 = M.c0;
-  if (M.interp0 == NTC_INTERP_LEARNED) {
-    // learned interpolation (Sec. 4.3.1): the four G0 taps concatenated
-    const ntc_level& L = M.lv[j];
-    const Taps t = bilinear_taps(x, y, wm, hm, L.g0_w, L.g0_h);
-#pragma unroll 1
-    for (int tp = 0; tp < 4; ++tp)
-      for (int ch = 0; ch < M.c0; ++ch) sink(tp * M.c0 + ch, grid_value(M, j, 0, t.cell[tp], ch, noise, nkey));
-    w0 = 4 * M.c0;
-  } else {
-    sample_grid(M, j, 0, x, y, wm, hm, noise, nkey, gs);
-#pragma unroll
-    for (int ch = 0; ch < kMaxGridCh; ++ch)
-      if (ch < M.c0) sink(ch, gs.acc[ch]);
-  }
-  sample_grid(M, j, 1, x, y, wm, hm, noise, nkey, gs);
-#pragma unroll
-  for (int ch = 0; ch < kMaxGridCh; ++ch)
-    if (ch < M.c1) sink(w0 + ch, gs.acc[ch]);
-  const int pe = w0 + M.c1;
-  positional_encoding(x, y, pe, sink);
-  sink(pe + 12, M.mips > 1 ? (float)m / (float)(M.mips - 1) : 0.f);
-  for (int i = pe + 13; i < M.k_in; ++i) sink(i, 0.f);
+  grid_features(M, 0, x, y, m, noise, nkey, sink);
+  grid_features(M, 1, x, y, m, noise, nkey, sink);
+  tail_features(M, x, y, m, sink);
 }
 
 // Level of detail of a training draw (Sec. 5.1) from the hashes of counters
@@ -421,25 +460,6 @@ __device__ __forceinline__ float act_grad(int act, float z) {
 }
 __device__ __forceinline__ float out_fwd(int out_act, float z) {
   return out_act == NTC_OUT_IDENTITY ? z : 1.f / (1.f + __expf(-z));
-}
-
-// Element idx of the third hidden layer's weights (hidden_layers == 3) as
-// float: FP32 or FP16.
-__device__ __forceinline__ float load_weight_h3(const ntc_material& M, int idx) {
-  if (M.precision == NTC_PREC_F16) return __half2float(static_cast<const __half*>(M.w_h3)[idx]);
-  return static_cast<const float*>(M.w_h3)[idx];
-}
-
-// Weight element l (0..2) at [o][i] as float, from the material's precision.
-__device__ __forceinline__ float load_weight(const ntc_material& M, int l, int idx) {
-  switch (M.precision) {
-    case NTC_PREC_F16: return __half2float(static_cast<const __half*>(M.w[l])[idx]);
-    case NTC_PREC_F8: {
-      const __nv_fp8_e4m3 v = static_cast<const __nv_fp8_e4m3*>(M.w[l])[idx];
-      return (float)v * M.scale[l];
-    }
-    default: return static_cast<const float*>(M.w[l])[idx];
-  }
 }
 
 }  // namespace ntc

@@ -1,9 +1,8 @@
-// FP32 CUDA-core form of the NTC hot path: random-access decode (nearest and
-// trilinear) and the fused forward + loss + backward of the optimisation
-// (Sec. 4.3-4.5, 5.1, 5.3).  One query / training texel per thread, the
-// material's weights staged once per CTA in shared memory, every activation
-// recomputed on chip (nothing but the per-tile operands of the weight-gradient
-// reduction touches memory).
+// FP32 CUDA-core form of the NTC hot path: random-access decode (nearest,
+// trilinear, stochastic) and the fused forward + loss + backward of the
+// optimisation (Sec. 4.3-4.5, 5.1, 5.3).  The MLP runs as register-tiled
+// FP32 matrix products on tiles of 32 queries / texels whose activations stay
+// in shared memory; every activation is recomputed on chip.
 #include "ntc_device.cuh"
 #include "ntc_internal.h"
 
@@ -11,221 +10,268 @@ namespace ntc {
 
 namespace {
 
-constexpr int kThreads = kTile;  // 128
+// ---------------------------------------------------------------------------
+// Decode.  A warp owns a tile of 32 queries.  Its input rows (and, in place,
+// the hidden rows) lie in shared memory unit-major, act[unit][kLd] with the
+// 32 queries contiguous, and lane (qg = lane / 8, ng = lane % 8) computes the
+// outputs n = ng + 8 j of queries 4 qg .. +3 and 16 + 4 qg .. +3: 64 FP32
+// accumulators for a 64-wide layer, four 16-byte shared loads per 64 FMAs.
+// The FMA chain of every output runs over k in order from the bias, so the
+// values are those of a plain loop.  kLd = 36 puts eight consecutive units
+// on disjoint banks for the 16-byte stores of a quarter-warp.
+// What bounds it: the FP32 FMA rate (78.4 TFLOP/s measured).  One thread per
+// query with every weight broadcast from shared memory (the form this
+// replaced) needed a 16-byte load per four FMAs and was bound by them:
+// a pass of 65,536 queries of a 256^2 x 8 material took 86 us against 31 now
+// (25 of them the host's share of a call).
+// ---------------------------------------------------------------------------
+constexpr int kLd = 36;         // floats per unit row: 32 queries + 4 of padding
+constexpr int kMaxWarps = 16;   // tiles in flight per CTA (one CTA per SM)
 
-// Shared-memory weights in float: W1^T [K][64] (input-major, for the
-// forward), W2 [64][64] and W3 [16][64] ([out][in]; W3 rows >= C are zero),
-// b1, b2, b3 (16), and with a third hidden layer Wh [64][64], bh.  Offsets in
-// floats, all multiples of 4.
+// Shared-memory weights of the decode, in floats: hidden layers [k][64] with
+// output n = ng + 8 j at 32 (j / 4) + 4 ng + j % 4, the output layer [64][16]
+// with n = ng + 8 j at 2 ng + j (rows >= C zero), biases, then one activation
+// region per warp (`rows` units and the 32 blend weights of trilinear taps).
 struct SW {
-  int w1t, w2, w3, b1, b2, b3, wh, bh, size;
+  int w1, w2, w3, b1, b2, b3, wh, bh, act, warp;
   bool h3;
   __host__ __device__ SW(int K, bool third) {
-    w1t = 0;
-    w2 = w1t + K * kHidden;
+    w1 = 0;
+    w2 = w1 + K * kHidden;
     w3 = w2 + kHidden * kHidden;
     b1 = w3 + kMaxC * kHidden;
     b2 = b1 + kHidden;
     b3 = b2 + kHidden;
     wh = b3 + kMaxC;
     bh = wh + (third ? kHidden * kHidden : 0);
-    size = bh + (third ? kHidden : 0);
+    act = bh + (third ? kHidden : 0);
+    warp = (K > kHidden ? K : kHidden) * kLd + 32;
     h3 = third;
   }
+  __host__ __device__ size_t bytes(int warps) const { return (size_t)(act + warps * warp) * 4; }
 };
+
+// Four consecutive inputs k .. k + 3 (k a multiple of 4) of row o of a
+// weight matrix [rows][ld] in the material's precision.
+__device__ __forceinline__ float4 weight4(const ntc_material& M, const void* w, float scale, int i) {
+  switch (M.precision) {
+    case NTC_PREC_F16: {
+      const uint2 v = __ldg(reinterpret_cast<const uint2*>(static_cast<const __half*>(w) + i));
+      union { uint32_t u; __half2 h; } a, b;
+      a.u = v.x;
+      b.u = v.y;
+      const float2 lo = __half22float2(a.h), hi = __half22float2(b.h);
+      return make_float4(lo.x, lo.y, hi.x, hi.y);
+    }
+    case NTC_PREC_F8: {
+      const __nv_fp8_e4m3* e = static_cast<const __nv_fp8_e4m3*>(w) + i;
+      return make_float4((float)e[0] * scale, (float)e[1] * scale, (float)e[2] * scale,
+                         (float)e[3] * scale);
+    }
+    default: return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(w) + i));
+  }
+}
+
+// Stage W [64][ld] so that place(o) + 64 k holds (o, k): lanes take
+// consecutive outputs, which `place` puts on different banks.
+template <class Place>
+__device__ __forceinline__ void stage_hidden(const ntc_material& M, const void* w, float scale,
+                                             int ld, float* dst, Place place) {
+  for (int i = threadIdx.x; i < kHidden * (ld / 4); i += blockDim.x) {
+    const int o = i & (kHidden - 1), k = 4 * (i >> 6);
+    const float4 v = weight4(M, w, scale, o * ld + k);
+    float* d = dst + place(o) + k * kHidden;
+    d[0] = v.x;
+    d[kHidden] = v.y;
+    d[2 * kHidden] = v.z;
+    d[3 * kHidden] = v.w;
+  }
+}
 
 __device__ void stage_weights(const ntc_material& M, const SW& L, float* s) {
   const int C = M.channels, K = M.k_in;
-  for (int i = threadIdx.x; i < kHidden * K; i += blockDim.x) {
-    const int o = i / K, k = i - o * K;
-    s[L.w1t + k * kHidden + o] = load_weight(M, 0, i);
+  const bool f8 = M.precision == NTC_PREC_F8;
+  auto place = [](int o) { return 32 * (o >> 5) + 4 * (o & 7) + ((o >> 3) & 3); };
+  stage_hidden(M, M.w[0], f8 ? M.scale[0] : 1.f, K, s + L.w1, place);
+  stage_hidden(M, M.w[1], f8 ? M.scale[1] : 1.f, kHidden, s + L.w2, place);
+  for (int i = threadIdx.x; i < kMaxC * (kHidden / 4); i += blockDim.x) {
+    const int c = i & (kMaxC - 1), k = 4 * (i >> 4);
+    const float4 v = c < C ? weight4(M, M.w[2], f8 ? M.scale[2] : 1.f, c * kHidden + k)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    float* d = s + L.w3 + 2 * (c & 7) + (c >> 3) + k * kMaxC;
+    d[0] = v.x;
+    d[kMaxC] = v.y;
+    d[2 * kMaxC] = v.z;
+    d[3 * kMaxC] = v.w;
   }
-  for (int i = threadIdx.x; i < kHidden * kHidden; i += blockDim.x) s[L.w2 + i] = load_weight(M, 1, i);
-  for (int i = threadIdx.x; i < kMaxC * kHidden; i += blockDim.x)
-    s[L.w3 + i] = (i / kHidden) < C ? load_weight(M, 2, i) : 0.f;
   for (int i = threadIdx.x; i < kHidden; i += blockDim.x) {
     s[L.b1 + i] = M.b[0][i];
     s[L.b2 + i] = M.b[1][i];
+    if (L.h3) s[L.bh + i] = M.b_h3[i];
   }
   for (int i = threadIdx.x; i < kMaxC; i += blockDim.x) s[L.b3 + i] = i < C ? M.b[2][i] : 0.f;
-  if (L.h3) {
-    for (int i = threadIdx.x; i < kHidden * kHidden; i += blockDim.x) s[L.wh + i] = load_weight_h3(M, i);
-    for (int i = threadIdx.x; i < kHidden; i += blockDim.x) s[L.bh + i] = M.b_h3[i];
-  }
+  if (L.h3) stage_hidden(M, M.w_h3, 1.f, kHidden, s + L.wh, place);
 }
 
-// Layer 1: z = W1 x + b1 with x a K-float row in shared memory (16-byte
-// aligned) and W1^T input-major: 64 independent accumulators per thread,
-// one broadcast float4 of weights per four FMAs.
-__device__ __forceinline__ void layer1(const float* __restrict__ w1t, const float* __restrict__ b1,
-                                       const float* __restrict__ xrow, int K, float (&z)[kHidden]) {
+// The lane's J outputs n = ng + 8 j (J = 8: a hidden layer, J = 2: the output
+// layer) of its eight queries: z[j][p] holds queries 4 qg + {0,1}, {2,3} and
+// 16 + 4 qg + {0,1}, {2,3}.
+template <int J>
+__device__ __forceinline__ void warp_dense(const float* __restrict__ W, const float* __restrict__ b,
+                                           const float* __restrict__ act, int K, int lane,
+                                           float2 (&z)[J][4]) {
+  const int ng = lane & 7, qg = lane >> 3;
 #pragma unroll
-  for (int o = 0; o < kHidden; ++o) z[o] = b1[o];
-#pragma unroll 1
-  for (int i = 0; i < K; i += 4) {
-    const float4 xv = *reinterpret_cast<const float4*>(xrow + i);
-    const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
+  for (int j = 0; j < J; ++j) {
+    const float bj = b[ng + 8 * j];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float* wr = w1t + (i + j) * kHidden;
+    for (int p = 0; p < 4; ++p) z[j][p] = make_float2(bj, bj);
+  }
+  const float* xp = act + 4 * qg;
+  const float* wp = W + (J == 8 ? 4 : 2) * ng;
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    const float4 xa = *reinterpret_cast<const float4*>(xp + k * kLd);
+    const float4 xb = *reinterpret_cast<const float4*>(xp + k * kLd + 16);
+    float w[J];
+    if constexpr (J == 8) {
+      const float4 w0 = *reinterpret_cast<const float4*>(wp + k * kHidden);
+      const float4 w1 = *reinterpret_cast<const float4*>(wp + k * kHidden + 32);
+      w[0] = w0.x; w[1] = w0.y; w[2] = w0.z; w[3] = w0.w;
+      w[4] = w1.x; w[5] = w1.y; w[6] = w1.z; w[7] = w1.w;
+    } else {
+      const float2 w0 = *reinterpret_cast<const float2*>(wp + k * kMaxC);
+      w[0] = w0.x; w[1] = w0.y;
+    }
 #pragma unroll
-      for (int o = 0; o < kHidden; o += 4) {
-        const float4 w = *reinterpret_cast<const float4*>(wr + o);
-        z[o] = fmaf(w.x, xs[j], z[o]);
-        z[o + 1] = fmaf(w.y, xs[j], z[o + 1]);
-        z[o + 2] = fmaf(w.z, xs[j], z[o + 2]);
-        z[o + 3] = fmaf(w.w, xs[j], z[o + 3]);
-      }
+    for (int j = 0; j < J; ++j) {
+      const float2 ww = make_float2(w[j], w[j]);
+      z[j][0] = __ffma2_rn(ww, make_float2(xa.x, xa.y), z[j][0]);
+      z[j][1] = __ffma2_rn(ww, make_float2(xa.z, xa.w), z[j][1]);
+      z[j][2] = __ffma2_rn(ww, make_float2(xb.x, xb.y), z[j][2]);
+      z[j][3] = __ffma2_rn(ww, make_float2(xb.z, xb.w), z[j][3]);
     }
   }
 }
 
-// y = W x + b for W [OUT][64] in shared memory, x in registers; four outputs
-// at a time so each thread carries four independent FMA chains.
-template <int OUT>
-__device__ __forceinline__ void dense64(const float* __restrict__ W, const float* __restrict__ b,
-                                        const float (&x)[kHidden], float (&y)[OUT]) {
+// act(z) of a hidden layer -> the warp's unit rows, once every lane has read
+// the layer's input.
+__device__ __forceinline__ void put_hidden(float* act, int lane, int fn, float2 (&z)[8][4]) {
+  __syncwarp();
+  float* p = act + (lane & 7) * kLd + 4 * (lane >> 3);
 #pragma unroll
-  for (int o = 0; o < OUT; o += 4) {
-    float a0 = b[o], a1 = b[o + 1], a2 = b[o + 2], a3 = b[o + 3];
+  for (int j = 0; j < 8; ++j) {
 #pragma unroll
-    for (int i = 0; i < kHidden; i += 4) {
-      const float4 w0 = *reinterpret_cast<const float4*>(W + (o + 0) * kHidden + i);
-      const float4 w1 = *reinterpret_cast<const float4*>(W + (o + 1) * kHidden + i);
-      const float4 w2 = *reinterpret_cast<const float4*>(W + (o + 2) * kHidden + i);
-      const float4 w3 = *reinterpret_cast<const float4*>(W + (o + 3) * kHidden + i);
-      a0 = fmaf(w0.x, x[i], a0); a0 = fmaf(w0.y, x[i + 1], a0);
-      a0 = fmaf(w0.z, x[i + 2], a0); a0 = fmaf(w0.w, x[i + 3], a0);
-      a1 = fmaf(w1.x, x[i], a1); a1 = fmaf(w1.y, x[i + 1], a1);
-      a1 = fmaf(w1.z, x[i + 2], a1); a1 = fmaf(w1.w, x[i + 3], a1);
-      a2 = fmaf(w2.x, x[i], a2); a2 = fmaf(w2.y, x[i + 1], a2);
-      a2 = fmaf(w2.z, x[i + 2], a2); a2 = fmaf(w2.w, x[i + 3], a2);
-      a3 = fmaf(w3.x, x[i], a3); a3 = fmaf(w3.y, x[i + 1], a3);
-      a3 = fmaf(w3.z, x[i + 2], a3); a3 = fmaf(w3.w, x[i + 3], a3);
+    for (int i = 0; i < 4; ++i) {
+      z[j][i].x = act_fwd(fn, z[j][i].x);
+      z[j][i].y = act_fwd(fn, z[j][i].y);
     }
-    y[o] = a0; y[o + 1] = a1; y[o + 2] = a2; y[o + 3] = a3;
+    *reinterpret_cast<float4*>(p + 8 * j * kLd) = make_float4(z[j][0].x, z[j][0].y, z[j][1].x, z[j][1].y);
+    *reinterpret_cast<float4*>(p + 8 * j * kLd + 16) = make_float4(z[j][2].x, z[j][2].y, z[j][3].x, z[j][3].y);
   }
+  __syncwarp();
 }
 
-// din = W^T d for W [OUT][64]: outer-product order over the outputs so that
-// every weight row is one broadcast read.
-template <int OUT>
-__device__ __forceinline__ void dense64_t(const float* __restrict__ W, const float (&d)[OUT],
-                                          float (&din)[kHidden]) {
-#pragma unroll
-  for (int i = 0; i < kHidden; ++i) din[i] = 0.f;
-#pragma unroll
-  for (int o = 0; o < OUT; ++o) {
-#pragma unroll
-    for (int i = 0; i < kHidden; i += 4) {
-      const float4 w = *reinterpret_cast<const float4*>(W + o * kHidden + i);
-      din[i] = fmaf(w.x, d[o], din[i]);
-      din[i + 1] = fmaf(w.y, d[o], din[i + 1]);
-      din[i + 2] = fmaf(w.z, d[o], din[i + 2]);
-      din[i + 3] = fmaf(w.w, d[o], din[i + 3]);
-    }
-  }
-}
-
-// Full decoder MLP on one input row held in shared memory.
-__device__ __forceinline__ void mlp_forward(const float* sw, const SW& L, const float* xrow, int K,
-                                            int act, int out_act, float (&y)[kMaxC]) {
-  float h1[kHidden];
-  layer1(sw + L.w1t, sw + L.b1, xrow, K, h1);
-#pragma unroll
-  for (int i = 0; i < kHidden; ++i) h1[i] = act_fwd(act, h1[i]);
-  float h2[kHidden];
-  dense64<kHidden>(sw + L.w2, sw + L.b2, h1, h2);
-#pragma unroll
-  for (int i = 0; i < kHidden; ++i) h2[i] = act_fwd(act, h2[i]);
-  if (L.h3) {
-    // third hidden layer (Sec. 4.4: activations on three layers)
-    dense64<kHidden>(sw + L.wh, sw + L.bh, h2, h1);
-#pragma unroll
-    for (int i = 0; i < kHidden; ++i) h2[i] = act_fwd(act, h1[i]);
-  }
-  dense64<kMaxC>(sw + L.w3, sw + L.b3, h2, y);
-#pragma unroll
-  for (int c = 0; c < kMaxC; ++c) y[c] = out_fwd(out_act, y[c]);
-}
-
-struct RowSink {
-  float* row;
-  __device__ __forceinline__ void operator()(int i, float v) const { row[i] = v; }
+// Input rows are written one query per lane: unit i of this lane's column.
+struct ColumnSink {
+  float* col;
+  __device__ __forceinline__ void operator()(int i, float v) const { col[i * kLd] = v; }
 };
 
-// Row stride of the per-thread input rows: K + 4 keeps rows 16-byte aligned
-// and makes a quarter-warp's float4 reads hit eight disjoint bank groups.
-__host__ __device__ __forceinline__ int row_stride(int K) { return K + 4; }
+// One output element of the decode.
+__device__ __forceinline__ void store_value(void* out, int out_dtype, int64_t e, float y) {
+  if (out_dtype == NTC_DTYPE_F32) static_cast<float*>(out)[e] = y;
+  else if (out_dtype == NTC_DTYPE_U8)
+    static_cast<uint8_t*>(out)[e] = (uint8_t)__float2uint_rn(__saturatef(y) * 255.f);
+  else static_cast<__half*>(out)[e] = __float2half_rn(y);
+}
 
-__global__ void __launch_bounds__(kThreads) decode_simt_kernel(
+__global__ void __launch_bounds__(32 * kMaxWarps, 1) decode_simt_kernel(
     const ntc_material M, const float* __restrict__ uvl, int64_t n, void* __restrict__ out,
     int out_dtype, int filter, int noise, uint64_t nkey, uint64_t jkey) {
   extern __shared__ __align__(16) float smem[];
   const int K = M.k_in, C = M.channels;
   const SW L(K, M.hidden_layers == 3);
-  float* sw = smem;
-  stage_weights(M, L, sw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  stage_weights(M, L, smem);
   __syncthreads();
-  RowSink sink{smem + L.size + threadIdx.x * row_stride(K)};
-  for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < n;
-       q += (int64_t)gridDim.x * kThreads) {
+  float* act = smem + L.act + warp * L.warp;
+  float* wtap = act + L.warp - 32;
+  ColumnSink sink{act + lane};
+  const int ng = lane & 7, qg = lane >> 3;
+  const bool tri = filter == NTC_FILTER_TRILINEAR;
+  const int64_t tiles = (n + 31) / 32;
+  for (int64_t t = blockIdx.x + (int64_t)warp * gridDim.x; t < tiles; t += (int64_t)gridDim.x * warps) {
+    // the lanes past the last query repeat it; their outputs are not stored
+    const int64_t q = min(t * 32 + lane, n - 1);
     const float u = uvl[3 * q], v = uvl[3 * q + 1], l = uvl[3 * q + 2];
-    float y[kMaxC];
-    if (filter == NTC_FILTER_NEAREST) {
-      int x, yy, m;
-      query_texel(M, u, v, l, x, yy, m);
-      featurize(M, x, yy, m, noise != 0, nkey, sink);
-      mlp_forward(sw, L, sink.row, K, M.act, M.out_act, y);
-    } else if (filter == NTC_FILTER_STOCHASTIC) {
-      const uint64_t h = splitmix64(jkey ^ (uint64_t)q);
-      const int m = stochastic_mip(l, M.mips, h);
-      const int x = stochastic_coord(u, mip_dim(M.width, m), (uint32_t)(h >> 40));
-      const int yy = stochastic_coord(v, mip_dim(M.height, m), (uint32_t)(h >> 16) & 0xFFFFFFu);
-      featurize(M, x, yy, m, false, 0, sink);
-      mlp_forward(sw, L, sink.row, K, M.act, M.out_act, y);
-    } else {
-      // software trilinear filtering (Sec. 5.3): 2x2 texels on two mips
-      const float lam = !(l >= 0.f) ? 0.f : fminf(l, (float)(M.mips - 1));
-      const int m0 = min((int)floorf(lam), M.mips - 1);
-      const int m1 = min(m0 + 1, M.mips - 1);
-      const float t = lam - (float)m0;
-#pragma unroll
-      for (int c = 0; c < kMaxC; ++c) y[c] = 0.f;
+    float2 y[2][4];
 #pragma unroll 1
-      for (int tap = 0; tap < 8; ++tap) {
+    for (int tap = 0; tap < (tri ? 8 : 1); ++tap) {
+      int x, yy, m;
+      if (filter == NTC_FILTER_NEAREST) {
+        query_texel(M, u, v, l, x, yy, m);
+      } else if (filter == NTC_FILTER_STOCHASTIC) {
+        const uint64_t h = splitmix64(jkey ^ (uint64_t)q);
+        m = stochastic_mip(l, M.mips, h);
+        x = stochastic_coord(u, mip_dim(M.width, m), (uint32_t)(h >> 40));
+        yy = stochastic_coord(v, mip_dim(M.height, m), (uint32_t)(h >> 16) & 0xFFFFFFu);
+      } else {
+        // software trilinear filtering (Sec. 5.3): 2x2 texels on two mips
+        const float lam = !(l >= 0.f) ? 0.f : fminf(l, (float)(M.mips - 1));
+        const int m0 = min((int)floorf(lam), M.mips - 1);
+        const int m1 = min(m0 + 1, M.mips - 1);
+        const float tl = lam - (float)m0;
         const int s = tap >> 2, dx = tap & 1, dy = (tap >> 1) & 1;
-        const int m = s ? m1 : m0;
-        const float wl = s ? t : 1.f - t;
+        m = s ? m1 : m0;
+        const float wl = s ? tl : 1.f - tl;
         const int wm = mip_dim(M.width, m), hm = mip_dim(M.height, m);
         const float px = u * (float)wm - 0.5f, py = v * (float)hm - 0.5f;
         const float fx0 = floorf(px), fy0 = floorf(py);
         const float fx = px - fx0, fy = py - fy0;
-        const int xx = (((int)fx0 + dx) % wm + wm) % wm, yv = (((int)fy0 + dy) % hm + hm) % hm;
-        const float w = wl * (dx ? fx : 1.f - fx) * (dy ? fy : 1.f - fy);
-        featurize(M, xx, yv, m, false, 0, sink);
-        float yt[kMaxC];
-        mlp_forward(sw, L, sink.row, K, M.act, M.out_act, yt);
-#pragma unroll
-        for (int c = 0; c < kMaxC; ++c) y[c] = fmaf(w, yt[c], y[c]);
+        x = (((int)fx0 + dx) % wm + wm) % wm;
+        yy = (((int)fy0 + dy) % hm + hm) % hm;
+        wtap[lane] = wl * (dx ? fx : 1.f - fx) * (dy ? fy : 1.f - fy);
       }
+      featurize(M, x, yy, m, noise != 0, nkey, sink);
+      __syncwarp();
+      float2 z[8][4];
+      warp_dense<8>(smem + L.w1, smem + L.b1, act, K, lane, z);
+      put_hidden(act, lane, M.act, z);
+      warp_dense<8>(smem + L.w2, smem + L.b2, act, kHidden, lane, z);
+      put_hidden(act, lane, M.act, z);
+      if (L.h3) {
+        // third hidden layer (Sec. 4.4: activations on three layers)
+        warp_dense<8>(smem + L.wh, smem + L.bh, act, kHidden, lane, z);
+        put_hidden(act, lane, M.act, z);
+      }
+      float2 o[2][4];
+      warp_dense<2>(smem + L.w3, smem + L.b3, act, kHidden, lane, o);
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const float2 yo = make_float2(out_fwd(M.out_act, o[j][p].x), out_fwd(M.out_act, o[j][p].y));
+          if (!tri) {
+            y[j][p] = yo;
+          } else {
+            const float2 w = *reinterpret_cast<const float2*>(wtap + 16 * (p >> 1) + 4 * qg + 2 * (p & 1));
+            const float2 y0 = tap ? y[j][p] : make_float2(0.f, 0.f);
+            y[j][p] = make_float2(fmaf(w.x, yo.x, y0.x), fmaf(w.y, yo.y, y0.y));
+          }
+        }
+      __syncwarp();  // the next tile's rows overwrite the activations
     }
-    if (out_dtype == NTC_DTYPE_F32) {
-      float* o = static_cast<float*>(out) + q * C;
 #pragma unroll
-      for (int c = 0; c < kMaxC; ++c)
-        if (c < C) o[c] = y[c];
-    } else if (out_dtype == NTC_DTYPE_U8) {
-      uint8_t* o = static_cast<uint8_t*>(out) + q * C;
+    for (int p = 0; p < 4; ++p)
 #pragma unroll
-      for (int c = 0; c < kMaxC; ++c)
-        if (c < C) o[c] = (uint8_t)__float2uint_rn(__saturatef(y[c]) * 255.f);
-    } else {
-      __half* o = static_cast<__half*>(out) + q * C;
-#pragma unroll
-      for (int c = 0; c < kMaxC; ++c)
-        if (c < C) o[c] = __float2half_rn(y[c]);
-    }
+      for (int e = 0; e < 2; ++e) {
+        const int64_t qo = t * 32 + 16 * (p >> 1) + 4 * qg + 2 * (p & 1) + e;
+        if (qo < n) {
+          if (ng < C) store_value(out, out_dtype, qo * C + ng, e ? y[0][p].y : y[0][p].x);
+          if (ng + 8 < C) store_value(out, out_dtype, qo * C + ng + 8, e ? y[1][p].y : y[1][p].x);
+        }
+      }
   }
 }
 
@@ -233,40 +279,46 @@ __global__ void __launch_bounds__(kThreads) decode_simt_kernel(
 // input (the feature row, act(Z1), act(Z2)) over the nearest decodes of the
 // queries, in FP32, reduced per warp and merged into amax[3] (float bits;
 // every value is non-negative, so the unsigned order is the float order).
-__global__ void __launch_bounds__(kThreads) f8_calib_kernel(const ntc_material M,
-                                                            const float* __restrict__ uvl,
-                                                            int64_t n, uint32_t* amax) {
+__global__ void __launch_bounds__(32 * kMaxWarps, 1) f8_calib_kernel(const ntc_material M,
+                                                                     const float* __restrict__ uvl,
+                                                                     int64_t n, uint32_t* amax) {
   extern __shared__ __align__(16) float smem[];
   const int K = M.k_in;
   const SW L(K, false);
-  float* sw = smem;
-  stage_weights(M, L, sw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  stage_weights(M, L, smem);
   __syncthreads();
-  RowSink sink{smem + L.size + threadIdx.x * row_stride(K)};
+  float* act = smem + L.act + warp * L.warp;
+  ColumnSink sink{act + lane};
   float mx[3] = {0.f, 0.f, 0.f};
-  for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < n;
-       q += (int64_t)gridDim.x * kThreads) {
+  auto merge = [](float& a, const float2 (&z)[8][4]) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int p = 0; p < 4; ++p) a = fmaxf(a, fmaxf(fabsf(z[j][p].x), fabsf(z[j][p].y)));
+  };
+  const int64_t tiles = (n + 31) / 32;
+  for (int64_t t = blockIdx.x + (int64_t)warp * gridDim.x; t < tiles; t += (int64_t)gridDim.x * warps) {
+    const int64_t q = min(t * 32 + lane, n - 1);  // the last query again past the end
     int x, yy, m;
     query_texel(M, uvl[3 * q], uvl[3 * q + 1], uvl[3 * q + 2], x, yy, m);
     featurize(M, x, yy, m, false, 0, sink);
-    for (int k = 0; k < K; ++k) mx[0] = fmaxf(mx[0], fabsf(sink.row[k]));
-    float h1[kHidden], h2[kHidden];
-    layer1(sw + L.w1t, sw + L.b1, sink.row, K, h1);
-#pragma unroll
-    for (int i = 0; i < kHidden; ++i) {
-      h1[i] = act_fwd(M.act, h1[i]);
-      mx[1] = fmaxf(mx[1], fabsf(h1[i]));
-    }
-    dense64<kHidden>(sw + L.w2, sw + L.b2, h1, h2);
-#pragma unroll
-    for (int i = 0; i < kHidden; ++i) mx[2] = fmaxf(mx[2], fabsf(act_fwd(M.act, h2[i])));
+    for (int k = 0; k < K; ++k) mx[0] = fmaxf(mx[0], fabsf(sink.col[k * kLd]));
+    __syncwarp();
+    float2 z[8][4];
+    warp_dense<8>(smem + L.w1, smem + L.b1, act, K, lane, z);
+    put_hidden(act, lane, M.act, z);
+    merge(mx[1], z);
+    warp_dense<8>(smem + L.w2, smem + L.b2, act, kHidden, lane, z);
+    put_hidden(act, lane, M.act, z);
+    merge(mx[2], z);
   }
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
     float v = mx[l];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&amax[l], __float_as_uint(v));
+    if (lane == 0) atomicMax(&amax[l], __float_as_uint(v));
   }
 }
 
@@ -289,274 +341,402 @@ __global__ void f8_scales_kernel(const uint32_t* amax, float* sa) {
 }
 
 // ---------------------------------------------------------------------------
-// Fused forward + loss + backward (Sec. 5.1): per 128-texel tile,
-//  A) per thread: texel, features (+noise), forward; the pre-activations Z1,
-//     Z2 and the output gradient D3 go to shared memory;
-//  C3) CTA: dW3 += D3^T act(Z2), db3;
-//  B1) per thread: D2 over Z2's row, D1 in registers, grid-gradient
-//      scatter-add of dX through the bilinear taps;
-//  C2) CTA: dW2 += D2^T act(Z1), db2;
-//  B2) per thread: D1 over Z1's row;
-//  C1) CTA: dW1 += D1^T X, db1.
-// Weight gradients accumulate in shared memory over all tiles of the CTA and
-// are flushed once with atomics.
+// Fused forward + loss + backward (Sec. 5.1).  A CTA of 128 threads takes
+// tiles of 32 texels; units lie unit-major in shared memory as in the decode,
+// and thread (qg, ng) computes outputs n = ng + 16 j (j < 4) of texels 4 qg ..
+// +3 of every product (16 accumulators).  Per tile:
+//   features -> X;  Z1, H1 = act(Z1);  Z2, H2;  Z3 -> loss, D3;
+//   dW3 += D3 H2^T, D2 = (W3^T D3) act'(Z2) over H2;
+//   dW2 += D2 H1^T, D1 = (W2^T D2) act'(Z1) over H1;
+//   dW1 += D1 X^T,  dX = W1^T D1 -> scatter-add through the taps.
+// act' stays in the registers of the thread that owns the unit; the weight
+// gradients stay in registers over all tiles of the CTA (72 per thread: 4x8
+// blocks of dW1 and dW2, 1x8 of dW3) and leave once, staged row-major, as
+// vector reductions.
+// What bounds it: for a batch of a few thousand texels the serial chain of
+// one tile, hence small tiles spread over all SMs, with the rows' features
+// split over the warps (G0, G1, the encoding and target, the taps).  Tiles
+// of 128 texels, one per thread, ran a 4,096-texel step of a 256^2 x 8
+// material on 32 CTAs in 118 us (all launches of the step) against 47 now.
 // ---------------------------------------------------------------------------
+constexpr int kBTile = 32;
+constexpr int kBThreads = 128;
+constexpr int kTapMeta = 112;  // bytes per texel: 8 cell addresses, 8 weights, padding
+
 struct SB {
-  SW w;
-  int g, x, z1, z2, d3, dx, red, size;
-  __host__ __device__ explicit SB(int K) : w(K, false) {
-    g = w.size;                                  // gradient accumulators, layout of w
-    x = g + w.size;                              // [128][K+4]
-    z1 = x + kTile * row_stride(K);              // [128][65]
-    z2 = z1 + kTile * (kHidden + 1);             // [128][65]
-    d3 = z2 + kTile * (kHidden + 1);             // [128][17]
-    dx = d3 + kTile * (kMaxC + 1);               // [128][K+1]: dX over the feature slots
-    red = dx + kTile * (K + 1);                  // [4]
+  int w1f, w2f, w3f, w1b, w2b, w3b, b1, b2, b3, x, h1, h2, d3, meta, red, size;
+  __host__ __device__ explicit SB(int K) {
+    w1f = 0;                               // [K][64], output n = ng + 16 j at 4 ng + j
+    w2f = w1f + K * kHidden;               // [64][64]
+    w3f = w2f + kHidden * kHidden;         // [64][16]
+    w1b = w3f + kMaxC * kHidden;           // transposed for the backward: [64 o][64 slots]
+    w2b = w1b + kHidden * kHidden;         // [64 o][64 i]
+    w3b = w2b + kHidden * kHidden;         // [16 c][64 i]
+    b1 = w3b + kMaxC * kHidden;
+    b2 = b1 + kHidden;
+    b3 = b2 + kHidden;
+    x = b3 + kMaxC;                        // unit-major tiles, kLd floats per unit
+    h1 = x + K * kLd;
+    h2 = h1 + kHidden * kLd;
+    d3 = h2 + kHidden * kLd;
+    meta = d3 + kMaxC * kLd;
+    red = meta + kBTile * kTapMeta / 4;    // [4]
     size = red + 4;
   }
 };
 
-__global__ void __launch_bounds__(kThreads, 1) backward_simt_kernel(const ntc_material M,
-                                                                    const BwdArgs A) {
+__device__ __forceinline__ int place16(int n) { return 4 * (n & 15) + (n >> 4); }
+
+// Row-major W [rows][ld] -> [row][64] with column i at place16(i): the
+// backward's operand (lanes take consecutive columns: different banks).
+__device__ __forceinline__ void stage_backward(const ntc_material& M, const void* w, float scale,
+                                               int rows, int ld, int live, float* dst) {
+  for (int i = threadIdx.x; i < rows * kHidden; i += blockDim.x) {
+    const int o = i >> 6, k = i & (kHidden - 1);
+    float v = 0.f;
+    if (o < live && k < ld) {
+      const int e = o * ld + k;
+      if (M.precision == NTC_PREC_F16) v = __half2float(static_cast<const __half*>(w)[e]);
+      else if (M.precision == NTC_PREC_F8) v = (float)static_cast<const __nv_fp8_e4m3*>(w)[e] * scale;
+      else v = __ldg(static_cast<const float*>(w) + e);
+    }
+    dst[o * kHidden + place16(k)] = v;
+  }
+}
+
+// z[j] += the thread's outputs ng + 16 j of its four texels, over `rows`
+// units of `in` ([unit][kLd]) against W [unit][64].
+__device__ __forceinline__ void tile_dense(const float* __restrict__ W, const float* __restrict__ in,
+                                           int rows, int ng, int qg, float2 (&z)[4][2]) {
+  const float* xp = in + 4 * qg;
+  const float* wp = W + 4 * ng;
+#pragma unroll 4
+  for (int k = 0; k < rows; ++k) {
+    const float4 x = *reinterpret_cast<const float4*>(xp + k * kLd);
+    const float4 w4 = *reinterpret_cast<const float4*>(wp + k * kHidden);
+    const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 ww = make_float2(w[j], w[j]);
+      z[j][0] = __ffma2_rn(ww, make_float2(x.x, x.y), z[j][0]);
+      z[j][1] = __ffma2_rn(ww, make_float2(x.z, x.w), z[j][1]);
+    }
+  }
+}
+__device__ __forceinline__ void put_units(float* dst, int ng, int qg, const float2 (&z)[4][2]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    *reinterpret_cast<float4*>(dst + (ng + 16 * j) * kLd + 4 * qg) =
+        make_float4(z[j][0].x, z[j][0].y, z[j][1].x, z[j][1].y);
+}
+// z -> act(z), keeping act'(z).
+__device__ __forceinline__ void activate(int fn, float2 (&z)[4][2], float2 (&g)[4][2]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      g[j][p] = make_float2(act_grad(fn, z[j][p].x), act_grad(fn, z[j][p].y));
+      z[j][p] = make_float2(act_fwd(fn, z[j][p].x), act_fwd(fn, z[j][p].y));
+    }
+}
+
+// acc[r][s] += sum over the 32 texels of d[og + 16 r] h[ig + 8 s] (rows of
+// units; s < cols / 8).
+template <int R>
+__device__ __forceinline__ void outer_acc(const float* __restrict__ d, const float* __restrict__ h,
+                                          int og, int ig, int cols, float (&acc)[R][8]) {
+#pragma unroll 1
+  for (int q = 0; q < kBTile; q += 4) {
+    float4 dv[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) dv[r] = *reinterpret_cast<const float4*>(d + (og + 16 * r) * kLd + q);
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+      if (8 * s < cols) {
+        const float4 hv = *reinterpret_cast<const float4*>(h + (ig + 8 * s) * kLd + q);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          acc[r][s] = fmaf(dv[r].x, hv.x, acc[r][s]);
+          acc[r][s] = fmaf(dv[r].y, hv.y, acc[r][s]);
+          acc[r][s] = fmaf(dv[r].z, hv.z, acc[r][s]);
+          acc[r][s] = fmaf(dv[r].w, hv.w, acc[r][s]);
+        }
+      }
+  }
+}
+__device__ __forceinline__ float row_sum(const float* __restrict__ d) {
+  float s = 0.f;
+#pragma unroll
+  for (int q = 0; q < kBTile; q += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(d + q);
+    s += (v.x + v.y) + (v.z + v.w);
+  }
+  return s;
+}
+
+// The staged row-major array `src` (n floats, a multiple of 4) times `gs`
+// into the gradient at `g`.
+__device__ __forceinline__ void flush_rows(float* g, const float* src, int n, float gs) {
+  if (!g) return;
+  if ((reinterpret_cast<uintptr_t>(g) & 15) == 0 && (n & 3) == 0) {
+    for (int i = threadIdx.x; i < n / 4; i += kBThreads) {
+      const float4 v = reinterpret_cast<const float4*>(src)[i];
+      atomicAdd(reinterpret_cast<float4*>(g) + i, make_float4(v.x * gs, v.y * gs, v.z * gs, v.w * gs));
+    }
+  } else {
+    for (int i = threadIdx.x; i < n; i += kBThreads) atomicAdd(g + i, src[i] * gs);
+  }
+}
+
+__global__ void __launch_bounds__(kBThreads, 2) backward_simt_kernel(const ntc_material M,
+                                                                     const BwdArgs A) {
   extern __shared__ __align__(16) float smem[];
   const int K = M.k_in, C = M.channels;
-  const int W0 = M.interp0 == NTC_INTERP_LEARNED ? 4 * M.c0 : M.c0;  // width of the G0 slots
-  const int F = W0 + M.c1;
+  const bool learned0 = M.interp0 == NTC_INTERP_LEARNED;
+  const int W0 = learned0 ? 4 * M.c0 : M.c0;  // width of the G0 slots
   const SB S(K);
-  float* sw = smem;
-  float* sg = smem + S.g;
-  stage_weights(M, S.w, sw);
-  for (int i = threadIdx.x; i < S.w.size; i += blockDim.x) sg[i] = 0.f;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ng = (lane & 7) + 8 * (warp & 1), qg = (lane >> 3) + 4 * (warp >> 1);
+  const int ig = lane & 7, og = (lane >> 3) + 4 * warp;
+  {
+    const bool f8 = M.precision == NTC_PREC_F8;
+    const float s1 = f8 ? M.scale[0] : 1.f, s2 = f8 ? M.scale[1] : 1.f, s3 = f8 ? M.scale[2] : 1.f;
+    stage_hidden(M, M.w[0], s1, K, smem + S.w1f, place16);
+    stage_hidden(M, M.w[1], s2, kHidden, smem + S.w2f, place16);
+    for (int i = tid; i < kMaxC * (kHidden / 4); i += kBThreads) {
+      const int c = i & (kMaxC - 1), k = 4 * (i >> 4);
+      const float4 v = c < C ? weight4(M, M.w[2], s3, c * kHidden + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float* d = smem + S.w3f + c + k * kMaxC;
+      d[0] = v.x;
+      d[kMaxC] = v.y;
+      d[2 * kMaxC] = v.z;
+      d[3 * kMaxC] = v.w;
+    }
+    stage_backward(M, M.w[0], s1, kHidden, K, kHidden, smem + S.w1b);
+    stage_backward(M, M.w[1], s2, kHidden, kHidden, kHidden, smem + S.w2b);
+    stage_backward(M, M.w[2], s3, kMaxC, kHidden, C, smem + S.w3b);
+    for (int i = tid; i < kHidden; i += kBThreads) {
+      smem[S.b1 + i] = M.b[0][i];
+      smem[S.b2 + i] = M.b[1][i];
+    }
+    if (tid < kMaxC) smem[S.b3 + tid] = tid < C ? M.b[2][tid] : 0.f;
+  }
   const int64_t step = A.step_dev ? *A.step_dev : A.noise_step;
   const uint64_t nkey = rng_key(A.noise_seed, noise_stream(step));
   const uint64_t skey = rng_key(A.sample_seed, sampler_stream(step));
-  float* xrow = smem + S.x + tid * row_stride(K);
-  float* z1row = smem + S.z1 + tid * (kHidden + 1);
-  float* z2row = smem + S.z2 + tid * (kHidden + 1);
-  float* d3row = smem + S.d3 + tid * (kMaxC + 1);
-  float* dxrow = smem + S.dx + tid * (K + 1);
-  RowSink sink{xrow};
+  float* X = smem + S.x;
+  float* H1 = smem + S.h1;
+  float* H2 = smem + S.h2;
+  float* D3 = smem + S.d3;
+  uint8_t* meta = reinterpret_cast<uint8_t*>(smem + S.meta);
+  float aw1[4][8] = {}, aw2[4][8] = {}, aw3[1][8] = {}, ab = 0.f, ab3 = 0.f;
   float loss_acc = 0.f;
-  __syncthreads();
 
-  for (int64_t base = (int64_t)blockIdx.x * kTile; base < A.n; base += (int64_t)gridDim.x * kTile) {
-    const int64_t i = base + tid;
-    const bool valid = i < A.n;
-    // ---- A: forward --------------------------------------------------------
-    int x = 0, y = 0, m = 0;
-    if (valid) {
-      if (A.uvl) query_texel(M, A.uvl[3 * i], A.uvl[3 * i + 1], A.uvl[3 * i + 2], x, y, m);
-      else sample_train_texel(A.crops != 0, skey, i, M.width, M.height, M.mips, x, y, m);
-    }
-    featurize(M, x, y, m, A.noise != 0, nkey, sink);
-    float d1[kHidden];  // h1 during the forward, dZ1 during the backward
-    layer1(sw + S.w.w1t, sw + S.w.b1, xrow, K, d1);
-#pragma unroll
-    for (int k = 0; k < kHidden; ++k) { z1row[k] = d1[k]; d1[k] = act_fwd(M.act, d1[k]); }
-    float z2[kHidden];
-    dense64<kHidden>(sw + S.w.w2, sw + S.w.b2, d1, z2);
-#pragma unroll
-    for (int k = 0; k < kHidden; ++k) { z2row[k] = z2[k]; z2[k] = act_fwd(M.act, z2[k]); }
-    float d3[kMaxC];
-    dense64<kMaxC>(sw + S.w.w3, sw + S.w.b3, z2, d3);
+  for (int64_t base = (int64_t)blockIdx.x * kBTile; base < A.n; base += (int64_t)gridDim.x * kBTile) {
+    // ---- texel (one per lane, the same in every warp) -> rows ----------------
     {
-      const int wm = mip_dim(M.width, m);
-      const uint8_t* trow = A.train ? A.target + A.tgt_off[m] + ((int64_t)y * wm + x) * C : nullptr;
+      const int64_t i = base + lane;
+      const bool valid = i < A.n;
+      int x = 0, y = 0, m = 0;
+      if (valid) {
+        if (A.uvl) query_texel(M, A.uvl[3 * i], A.uvl[3 * i + 1], A.uvl[3 * i + 2], x, y, m);
+        else sample_train_texel(A.crops != 0, skey, i, M.width, M.height, M.mips, x, y, m);
+      }
+      ColumnSink sink{X + lane};
+      if (warp < 2) {
+        grid_features(M, warp, x, y, m, A.noise != 0, nkey, sink);
+      } else if (warp == 2) {
+        tail_features(M, x, y, m, sink);
+        // the target bytes (as floats) or the upstream gradient, in D3's place
+        const int wm = mip_dim(M.width, m);
+        const uint8_t* trow = A.train ? A.target + A.tgt_off[m] + ((int64_t)y * wm + x) * C : nullptr;
+#pragma unroll 4
+        for (int c = 0; c < kMaxC; ++c)
+          D3[c * kLd + lane] = valid && c < C ? (A.train ? (float)trow[c] : A.dout[i * C + c]) : 0.f;
+      } else {
+        // cell addresses and weights of the texel's taps in both grids
+        float** ga = reinterpret_cast<float**>(meta + lane * kTapMeta);
+        float* wt = reinterpret_cast<float*>(meta + lane * kTapMeta + 64);
+        const int j = level_of_mip(m, M.levels);
+        const int wm = mip_dim(M.width, m), hm = mip_dim(M.height, m);
+        const ntc_level& Lv = M.lv[j];
 #pragma unroll
-      for (int c = 0; c < kMaxC; ++c) {
+        for (int k = 0; k < 2; ++k) {
+          float* g = k ? A.g.grid1[j] : A.g.grid0[j];
+          const Taps t = bilinear_taps(x, y, wm, hm, k ? Lv.g1_w : Lv.g0_w, k ? Lv.g1_h : Lv.g0_h);
+#pragma unroll
+          for (int tp = 0; tp < 4; ++tp) {
+            ga[4 * k + tp] = g && valid ? g + (size_t)t.cell[tp] * (k ? M.c1 : M.c0) : nullptr;
+            wt[4 * k + tp] = (k == 0 && learned0 ? 1.f : t.w[tp]) * A.grad_scale;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // ---- forward -------------------------------------------------------------
+    float2 z[4][2], g1[4][2], g2[4][2];
+    auto bias = [&](const float* b) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float v = b ? b[ng + 16 * j] : 0.f;
+        z[j][0] = z[j][1] = make_float2(v, v);
+      }
+    };
+    bias(smem + S.b1);
+    tile_dense(smem + S.w1f, X, K, ng, qg, z);
+    activate(M.act, z, g1);
+    put_units(H1, ng, qg, z);
+    __syncthreads();
+    bias(smem + S.b2);
+    tile_dense(smem + S.w2f, H1, kHidden, ng, qg, z);
+    activate(M.act, z, g2);
+    put_units(H2, ng, qg, z);
+    __syncthreads();
+    {
+      // output channel ng of four texels; loss and D3
+      float o[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[e] = smem[S.b3 + ng];
+#pragma unroll 4
+      for (int k = 0; k < kHidden; ++k) {
+        const float4 h = *reinterpret_cast<const float4*>(H2 + k * kLd + 4 * qg);
+        const float w = smem[S.w3f + k * kMaxC + ng];
+        o[0] = fmaf(w, h.x, o[0]);
+        o[1] = fmaf(w, h.y, o[1]);
+        o[2] = fmaf(w, h.z, o[2]);
+        o[3] = fmaf(w, h.w, o[3]);
+      }
+      float4* dp = reinterpret_cast<float4*>(D3 + ng * kLd + 4 * qg);
+      const float4 t4 = *dp;
+      const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
         float g = 0.f;
-        if (valid && c < C) {
-          const float yc = out_fwd(M.out_act, d3[c]);
+        if (base + 4 * qg + e < A.n && ng < C) {
+          const float yc = out_fwd(M.out_act, o[e]);
           float dy;
           if (A.train) {
-            const float e = yc - (float)trow[c] * (1.f / 255.f);
-            loss_acc = fmaf(e, e, loss_acc);
-            dy = 2.f * e;
+            const float er = yc - tv[e] * (1.f / 255.f);
+            loss_acc = fmaf(er, er, loss_acc);
+            dy = 2.f * er;
           } else {
-            dy = A.dout[i * C + c];
+            dy = tv[e];
           }
           g = M.out_act == NTC_OUT_IDENTITY ? dy : dy * yc * (1.f - yc);
         }
-        d3[c] = g;
-        d3row[c] = g;
+        o[e] = g;
       }
+      *dp = make_float4(o[0], o[1], o[2], o[3]);
     }
     __syncthreads();
-    // ---- C3: dW3 += D3^T act(Z2), db3 -----------------------------------
-    {
-      const int c0 = 4 * (tid & 3), i0 = 2 * (tid >> 2);
-      float acc[4][2] = {};
-      float accb = 0.f;
-#pragma unroll 4
-      for (int b = 0; b < kTile; ++b) {
-        const float* zr = smem + S.z2 + b * (kHidden + 1);
-        const float* dr = smem + S.d3 + b * (kMaxC + 1);
-        const float h0 = act_fwd(M.act, zr[i0]), h1 = act_fwd(M.act, zr[i0 + 1]);
+    // ---- output layer: dW3, db3, D2 over H2 ------------------------------------
+    outer_acc<1>(D3, H2, og, ig, kHidden, aw3);
+    if (tid < kMaxC) ab3 += row_sum(D3 + tid * kLd);
+    bias(nullptr);
+    tile_dense(smem + S.w3b, D3, kMaxC, ng, qg, z);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          acc[r][0] = fmaf(dr[c0 + r], h0, acc[r][0]);
-          acc[r][1] = fmaf(dr[c0 + r], h1, acc[r][1]);
-        }
-        if (tid < kMaxC) accb += dr[tid];
-      }
+    for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        sg[S.w.w3 + (c0 + r) * kHidden + i0] += acc[r][0];
-        sg[S.w.w3 + (c0 + r) * kHidden + i0 + 1] += acc[r][1];
-      }
-      if (tid < kMaxC) sg[S.w.b3 + tid] += accb;
-    }
-    // ---- B1: D2 over Z2's row, D1 in registers, grid scatter ------------
-    {
-      float dh[kHidden];
-      dense64_t<kMaxC>(sw + S.w.w3, d3, dh);
-#pragma unroll
-      for (int k = 0; k < kHidden; ++k) dh[k] *= act_grad(M.act, z2row[k]);
-      __syncthreads();  // every thread is done reading Z2 (C3)
-#pragma unroll
-      for (int k = 0; k < kHidden; ++k) z2row[k] = dh[k];
-      dense64_t<kHidden>(sw + S.w.w2, dh, d1);
-#pragma unroll
-      for (int k = 0; k < kHidden; ++k) d1[k] *= act_grad(M.act, z1row[k]);
-    }
-    if (A.grids && valid) {
-      // dX = W1^T D1 over the feature slots (through shared memory, so the
-      // runtime offsets of the G0 / G1 slots need no register indexing)
-      const float* w1t = sw + S.w.w1t;
-#pragma unroll 1
-      for (int s = 0; s < F; ++s) {
-        float a = 0.f;
-#pragma unroll
-        for (int o = 0; o < kHidden; o += 4) {
-          const float4 w = *reinterpret_cast<const float4*>(w1t + s * kHidden + o);
-          a = fmaf(w.x, d1[o], a);
-          a = fmaf(w.y, d1[o + 1], a);
-          a = fmaf(w.z, d1[o + 2], a);
-          a = fmaf(w.w, d1[o + 3], a);
-        }
-        dxrow[s] = a;
-      }
-      const int j = level_of_mip(m, M.levels);
-      const int wm = mip_dim(M.width, m), hm = mip_dim(M.height, m);
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const ntc_level& Lv = M.lv[j];
-        float* g = k ? A.g.grid1[j] : A.g.grid0[j];
-        if (!g) continue;
-        const int c = k ? M.c1 : M.c0;
-        const bool learned = k == 0 && W0 != M.c0;
-        const Taps t = bilinear_taps(x, y, wm, hm, k ? Lv.g1_w : Lv.g0_w, k ? Lv.g1_h : Lv.g0_h);
-#pragma unroll
-        for (int tp = 0; tp < 4; ++tp) {
-          // bilinear: the tap's weight on the shared slots; learned
-          // interpolation: the tap's own slots with weight 1
-          const float* dk = dxrow + (k ? W0 : (learned ? tp * c : 0));
-          const float wgt = (learned ? 1.f : t.w[tp]) * A.grad_scale;
-          float* gp = g + (size_t)t.cell[tp] * c;
-          if ((c & 3) == 0) {
-            for (int c4 = 0; 4 * c4 < c; ++c4)
-              atomicAdd(reinterpret_cast<float4*>(gp) + c4,
-                        make_float4(dk[4 * c4] * wgt, dk[4 * c4 + 1] * wgt, dk[4 * c4 + 2] * wgt,
-                                    dk[4 * c4 + 3] * wgt));
-          } else {
-            for (int ch = 0; ch < c; ++ch) atomicAdd(gp + ch, dk[ch] * wgt);
-          }
-        }
-      }
-    }
-    __syncthreads();  // D2 complete in Z2's rows
-    // ---- C2: dW2 += D2^T act(Z1), db2 -----------------------------------
-    {
-      const int o0 = 4 * (tid & 15), i0 = 8 * (tid >> 4);
-      float acc[4][8] = {};
-      float accb = 0.f;
-#pragma unroll 2
-      for (int b = 0; b < kTile; ++b) {
-        const float* zr = smem + S.z1 + b * (kHidden + 1);
-        const float* dr = smem + S.z2 + b * (kHidden + 1);
-        float h[8];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) h[s] = act_fwd(M.act, zr[i0 + s]);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float d = dr[o0 + r];
-#pragma unroll
-          for (int s = 0; s < 8; ++s) acc[r][s] = fmaf(d, h[s], acc[r][s]);
-        }
-        if (tid < kHidden) accb += dr[tid];
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int s = 0; s < 8; ++s) sg[S.w.w2 + (o0 + r) * kHidden + i0 + s] += acc[r][s];
-      if (tid < kHidden) sg[S.w.b2 + tid] += accb;
-    }
-    __syncthreads();  // Z1 no longer read
-    // ---- B2: D1 over Z1's row ----------------------------------------------
-#pragma unroll
-    for (int k = 0; k < kHidden; ++k) z1row[k] = d1[k];
+      for (int p = 0; p < 2; ++p) z[j][p] = make_float2(z[j][p].x * g2[j][p].x, z[j][p].y * g2[j][p].y);
+    __syncthreads();  // H2 read
+    put_units(H2, ng, qg, z);
     __syncthreads();
-    // ---- C1: dW1 += D1^T X (4x8 output blocks), db1 ------------------------
-    {
-      const int nblk = (kHidden / 4) * (K / 8);
-      for (int blk = tid; blk < nblk; blk += kThreads) {
-        const int o0 = 4 * (blk & 15), i0 = 8 * (blk >> 4);
-        float acc[4][8] = {};
+    // ---- layer 2: dW2, db2, D1 over H1 -----------------------------------------
+    outer_acc<4>(H2, H1, og, ig, kHidden, aw2);
+    if (tid >= kHidden) ab += row_sum(H2 + (tid - kHidden) * kLd);
+    bias(nullptr);
+    tile_dense(smem + S.w2b, H2, kHidden, ng, qg, z);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) z[j][p] = make_float2(z[j][p].x * g1[j][p].x, z[j][p].y * g1[j][p].y);
+    __syncthreads();  // H1 and D2 read
+    put_units(H1, ng, qg, z);
+    __syncthreads();
+    // ---- layer 1: dW1, db1, dX (over D2) ----------------------------------------
+    outer_acc<4>(H1, X, og, ig, K, aw1);
+    if (tid < kHidden) ab += row_sum(H1 + tid * kLd);
+    if (A.grids) {
+      bias(nullptr);
+      tile_dense(smem + S.w1b, H1, kHidden, ng, qg, z);
+      put_units(H2, ng, qg, z);
+      __syncthreads();
+      // each warp scatters eight texels: lane j adds grid j / 16, tap
+      // (j / 4) % 4, four channels at a time, so the four lanes of a tap
+      // reduce 64 consecutive bytes of one cell
+      const int k = lane >> 4, slot = lane >> 2, qd = lane & 3;
+      const int c = k ? M.c1 : M.c0;
+      const int col = k ? W0 : (learned0 ? (slot & 3) * c : 0);
+      const float* dx = H2 + col * kLd;
 #pragma unroll 2
-        for (int b = 0; b < kTile; ++b) {
-          const float* xr = smem + S.x + b * row_stride(K);
-          const float* dr = smem + S.z1 + b * (kHidden + 1);
-          const float4 xa = *reinterpret_cast<const float4*>(xr + i0);
-          const float4 xb = *reinterpret_cast<const float4*>(xr + i0 + 4);
-          const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const float d = dr[o0 + r];
-#pragma unroll
-            for (int s = 0; s < 8; ++s) acc[r][s] = fmaf(d, xv[s], acc[r][s]);
-          }
+      for (int t = 8 * warp; t < 8 * warp + 8; ++t) {
+        float* const ga = *reinterpret_cast<float* const*>(meta + t * kTapMeta + 8 * slot);
+        if (!ga) continue;
+        const float w = *reinterpret_cast<const float*>(meta + t * kTapMeta + 64 + 4 * slot);
+        if ((c & 3) == 0) {
+          for (int ch = 4 * qd; ch < c; ch += 16)
+            atomicAdd(reinterpret_cast<float4*>(ga + ch),
+                      make_float4(dx[ch * kLd + t] * w, dx[(ch + 1) * kLd + t] * w,
+                                  dx[(ch + 2) * kLd + t] * w, dx[(ch + 3) * kLd + t] * w));
+        } else {
+          for (int ch = qd; ch < c; ch += 4) atomicAdd(ga + ch, dx[ch * kLd + t] * w);
         }
-        // dW1 is [64][K] row-major in the accumulator (the flush layout)
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int s = 0; s < 8; ++s) sg[S.w.w1t + (o0 + r) * K + i0 + s] += acc[r][s];
-      }
-      if (tid < kHidden) {
-        float accb = 0.f;
-        for (int b = 0; b < kTile; ++b) accb += smem[S.z1 + b * (kHidden + 1) + tid];
-        sg[S.w.b1 + tid] += accb;
       }
     }
     __syncthreads();  // tile buffers free
   }
 
-  // ---- flush the CTA's weight gradients and loss ---------------------------
+  // ---- flush: the CTA's weight gradients row-major over the weights' place ------
   const float gs = A.grad_scale;
-  if (A.g.w[0])
-    for (int i = tid; i < kHidden * K; i += blockDim.x) atomicAdd(A.g.w[0] + i, sg[S.w.w1t + i] * gs);
-  if (A.g.w[1])
-    for (int i = tid; i < kHidden * kHidden; i += blockDim.x)
-      atomicAdd(A.g.w[1] + i, sg[S.w.w2 + i] * gs);
-  if (A.g.w[2])
-    for (int i = tid; i < C * kHidden; i += blockDim.x) atomicAdd(A.g.w[2] + i, sg[S.w.w3 + i] * gs);
-  if (A.g.b[0])
-    for (int i = tid; i < kHidden; i += blockDim.x) atomicAdd(A.g.b[0] + i, sg[S.w.b1 + i] * gs);
-  if (A.g.b[1])
-    for (int i = tid; i < kHidden; i += blockDim.x) atomicAdd(A.g.b[1] + i, sg[S.w.b2 + i] * gs);
-  if (A.g.b[2])
-    for (int i = tid; i < C; i += blockDim.x) atomicAdd(A.g.b[2] + i, sg[S.w.b3 + i] * gs);
+  float* f1 = smem;                        // [64][K]
+  float* f2 = f1 + kHidden * K;            // [64][64]
+  float* f3 = f2 + kHidden * kHidden;      // [16][64]
+  float* fb = f3 + kMaxC * kHidden;        // db1, db2, db3
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (8 * s < K) f1[(og + 16 * r) * K + ig + 8 * s] = aw1[r][s];
+      f2[(og + 16 * r) * kHidden + ig + 8 * s] = aw2[r][s];
+    }
+    f3[og * kHidden + ig + 8 * s] = aw3[0][s];
+  }
+  fb[tid] = ab;
+  if (tid < kMaxC) fb[2 * kHidden + tid] = ab3;
+  __syncthreads();
+  flush_rows(A.g.w[0], f1, kHidden * K, gs);
+  flush_rows(A.g.w[1], f2, kHidden * kHidden, gs);
+  flush_rows(A.g.w[2], f3, C * kHidden, gs);
+  flush_rows(A.g.b[0], fb, kHidden, gs);
+  flush_rows(A.g.b[1], fb + kHidden, kHidden, gs);
+  flush_rows(A.g.b[2], fb + 2 * kHidden, C, gs);
   if (A.train && A.loss) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
     float* red = smem + S.red;
-    if ((tid & 31) == 0) red[tid >> 5] = loss_acc;
+    if (lane == 0) red[warp] = loss_acc;
     __syncthreads();
     if (tid == 0) atomicAdd(A.loss, (red[0] + red[1] + red[2] + red[3]) * A.loss_scale);
   }
 }
 
+}  // namespace
+
+namespace {
+// Warps per CTA of the tiled forward: the most (16, 12, 8 or 4) whose
+// activations fit beside the weights (16 up to K = 64, 12 at K = 96 with two
+// hidden layers, 8 at K = 128).
+int simt_warps(const SW& L) {
+  for (int w = kMaxWarps; w > 4; w -= 4)
+    if (L.bytes(w) <= 227 * 1024) return w;
+  return 4;
+}
+// One CTA per SM; tile t goes to CTA t mod grid, so a call with fewer tiles
+// than warps spreads over all SMs.
+int simt_grid(int64_t n) {
+  const int64_t tiles = (n + 31) / 32, cap = sm_count();
+  return (int)(tiles < cap ? tiles : cap);
+}
 }  // namespace
 
 cudaError_t launch_decode_simt(const ntc_material& m, const float* uvl, int64_t n, void* out,
@@ -566,18 +746,13 @@ cudaError_t launch_decode_simt(const ntc_material& m, const float* uvl, int64_t 
   const uint64_t nkey = rng_key(noise_seed, noise_stream(noise_step));
   const uint64_t jkey = jitter_key(noise_seed, noise_step);
   const SW L(m.k_in, m.hidden_layers == 3);
-  const size_t smem = (size_t)(L.size + kThreads * row_stride(m.k_in)) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(decode_simt_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int warps = simt_warps(L);
+  const size_t smem = L.bytes(warps);
+  const cudaError_t e = cudaFuncSetAttribute(
+      decode_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_simt_kernel, kThreads, smem);
-  if (e != cudaSuccess) return e;
-  const int64_t tiles = (n + kThreads - 1) / kThreads;
-  const int64_t cap = (int64_t)sm_count() * (per_sm > 0 ? per_sm : 1);
-  const int grid = (int)(tiles < cap ? tiles : cap);
-  decode_simt_kernel<<<grid, kThreads, smem, s>>>(m, uvl, n, out, out_dtype, filter, noise, nkey,
-                                                  jkey);
+  decode_simt_kernel<<<simt_grid(n), 32 * warps, smem, s>>>(m, uvl, n, out, out_dtype, filter, noise,
+                                                            nkey, jkey);
   return cudaGetLastError();
 }
 
@@ -587,12 +762,11 @@ cudaError_t launch_f8_calibrate(const ntc_material& m, const float* uvl, int64_t
   if (e != cudaSuccess) return e;
   if (n > 0) {
     const SW L(m.k_in, false);
-    const size_t smem = (size_t)(L.size + kThreads * row_stride(m.k_in)) * sizeof(float);
+    const int warps = simt_warps(L);
+    const size_t smem = L.bytes(warps);
     e = cudaFuncSetAttribute(f8_calib_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int64_t tiles = (n + kThreads - 1) / kThreads;
-    const int64_t cap = (int64_t)sm_count() * 4;
-    f8_calib_kernel<<<(int)(tiles < cap ? tiles : cap), kThreads, smem, s>>>(m, uvl, n, amax);
+    f8_calib_kernel<<<simt_grid(n), 32 * warps, smem, s>>>(m, uvl, n, amax);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -607,10 +781,10 @@ cudaError_t launch_backward_simt(const ntc_material& m, const BwdArgs& a, cudaSt
   cudaError_t e = cudaFuncSetAttribute(backward_simt_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int64_t tiles = (a.n + kTile - 1) / kTile;
-  const int64_t cap = sm_count();
+  const int64_t tiles = (a.n + kBTile - 1) / kBTile;
+  const int64_t cap = 2 * (int64_t)sm_count();
   const int grid = (int)(tiles < cap ? tiles : cap);
-  backward_simt_kernel<<<grid, kThreads, smem, s>>>(m, a);
+  backward_simt_kernel<<<grid, kBThreads, smem, s>>>(m, a);
   return cudaGetLastError();
 }
 

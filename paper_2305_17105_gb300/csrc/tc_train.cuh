@@ -702,7 +702,7 @@ __device__ __forceinline__ void learned_g0(const ntc_material& M, const TPlan& P
     for (int tp = 0; tp < 4; ++tp)
       for (int ch = 0; ch < c; ++ch)
         put_half(W, P, row, tp * c + ch,
-                 valid ? grid_value(M, j, 0, t.cell[tp], ch, noise, nkey) : 0.f);
+                 valid ? grid_value<true>(M, j, 0, t.cell[tp], ch, noise, nkey) : 0.f);
   }
   for (int s = P.w0; s < 8 * P.f0; ++s) put_half(W, P, row, s, 0.f);
 }
@@ -967,7 +967,7 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
         if (!noise_on && (ck & 3) == 0 && ck <= kFastGridCh)
           sample_grid_f32x4(M, j, k, x, y, wm, hm, gs, use_copy ? (k ? A.noisy1[j] : A.noisy0[j]) : nullptr);
         else
-          sample_grid(M, j, k, x, y, wm, hm, noise_on && valid, nkey, gs);
+          sample_grid<true>(M, j, k, x, y, wm, hm, noise_on && valid, nkey, gs);
         const int g0 = k ? P.f0 : 0, ng = k ? P.f1 : P.f0;
 #pragma unroll
         for (int g = 0; g < kGridPad / 8; ++g)
