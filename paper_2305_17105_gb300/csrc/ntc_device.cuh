@@ -83,6 +83,10 @@ __device__ __forceinline__ void query_texel(const ntc_material& M, float u, floa
 __host__ __device__ __forceinline__ uint64_t jitter_key(uint64_t seed, int64_t step) {
   return rng_key(seed, ((uint64_t)step << 2) | 2u);
 }
+// Texel index i of a repeating texture, wrapped into [0, w).  Mip sides are
+// powers of two, so the (floored) remainder is a mask: the two integer
+// divisions of i mod w cost about 40 instructions each.
+__device__ __forceinline__ int wrap_texel(int i, int w) { return i & (w - 1); }
 __device__ __forceinline__ int stochastic_mip(float lod, int mips, uint64_t h) {
   const float xl = (float)(uint32_t)(h & 0xFFFFu) * (1.f / 65536.f);
   const float l = !(lod >= 0.f) ? 0.f : fminf(lod, (float)(mips - 1));
@@ -92,8 +96,7 @@ __device__ __forceinline__ int stochastic_coord(float u, int w, uint32_t b24) {
   const float xi = (float)b24 * (1.f / 16777216.f);
   const float uc = fminf(fmaxf(u == u ? u : 0.f, -16384.f), 16384.f);
   const float p = __fadd_rn(__fadd_rn(__fmul_rn(uc, (float)w), -0.5f), xi);
-  const int i = (int)floorf(p);
-  return (i % w + w) % w;
+  return wrap_texel((int)floorf(p), w);
 }
 
 // Bilinear taps of a gw x gh grid for texel (x, y) of a wm x hm mip

@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) decode_simt_kernel(
         const float px = u * (float)wm - 0.5f, py = v * (float)hm - 0.5f;
         const float fx0 = floorf(px), fy0 = floorf(py);
         const float fx = px - fx0, fy = py - fy0;
-        x = (((int)fx0 + dx) % wm + wm) % wm;
-        yy = (((int)fy0 + dy) % hm + hm) % hm;
+        x = wrap_texel((int)fx0 + dx, wm);
+        yy = wrap_texel((int)fy0 + dy, hm);
         wtap[lane] = wl * (dx ? fx : 1.f - fx) * (dy ? fy : 1.f - fy);
       }
       featurize(M, x, yy, m, noise != 0, nkey, sink);

@@ -185,16 +185,11 @@ __global__ void __launch_bounds__(kRows* kNWG, 1) decode_tc_kernel(
       yv[c] = M.out_act == NTC_OUT_IDENTITY ? z : fmaf(0.5f, tc::tanh_fast(z), 0.5f);
     }
     if (tri) {
-#pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        float s = yv[c] * wtap;
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
-        s += __shfl_xor_sync(0xffffffffu, s, 2);
-        s += __shfl_xor_sync(0xffffffffu, s, 4);
-        yv[c] = s;
-      }
+      const int c = blend_taps(yv, wtap, row);
+      if (valid) store_pair(out, out_dtype, q * C, C, c, yv[0], yv[1]);
+    } else if (valid) {
+      store_texel(out, out_dtype, q, C, yv);
     }
-    if (valid && (!tri || (row & 7) == 0)) store_texel(out, out_dtype, q, C, yv);
     // the next tile's layer 1 overwrites D: every row must have read it
     tc::bar_sync(bar_id, kRows);
     if (*abort_flag) { aborted = true; break; }

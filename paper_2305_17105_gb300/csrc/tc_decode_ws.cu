@@ -263,38 +263,15 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_batched_kernel(
       tc::tmem_ld_wait();
       tc::fence_before_sync();
       out_activate(yv, m_oact);
-      if (tri) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          float s = yv[c] * wtap;
-          s += __shfl_xor_sync(0xffffffffu, s, 1);
-          s += __shfl_xor_sync(0xffffffffu, s, 2);
-          s += __shfl_xor_sync(0xffffffffu, s, 4);
-          yv[c] = s;
-        }
-      }
       const int C = m_C;
-      if (valid && (!tri || (row & 7) == 0)) {
-        // vector stores need the material's output block 16-byte aligned
+      if (tri) {
+        const int c = blend_taps(yv, wtap, row);
+        if (valid) store_pair(out, out_dtype, obase + (int64_t)ql * C, C, c, yv[0], yv[1]);
+      } else if (valid) {
+        // vectors as wide as the start of the material's output block allows
         const int eb = out_dtype == NTC_DTYPE_U8 ? 1 : (out_dtype == NTC_DTYPE_F16 ? 2 : 4);
-        if (((obase * eb) & 15) == 0) {
-          store_texel(static_cast<uint8_t*>(out) + obase * eb, out_dtype, ql, C, yv);
-        } else if (out_dtype == NTC_DTYPE_U8) {
-          uint8_t* o = static_cast<uint8_t*>(out) + obase + (int64_t)ql * C;
-#pragma unroll
-          for (int c = 0; c < 16; ++c)
-            if (c < C) o[c] = (uint8_t)__float2uint_rn(__saturatef(yv[c]) * 255.f);
-        } else if (out_dtype == NTC_DTYPE_F16) {
-          __half* o = static_cast<__half*>(out) + obase + (int64_t)ql * C;
-#pragma unroll
-          for (int c = 0; c < 16; ++c)
-            if (c < C) o[c] = __float2half_rn(yv[c]);
-        } else {
-          float* o = static_cast<float*>(out) + obase + (int64_t)ql * C;
-#pragma unroll
-          for (int c = 0; c < 16; ++c)
-            if (c < C) o[c] = yv[c];
-        }
+        store_texel_at(static_cast<uint8_t*>(out) + obase * eb, (int)(obase * eb) & 15, out_dtype,
+                       (int64_t)ql * C, C, yv);
       }
       if (*abort_flag) break;
       // a material boundary: every MMA of this warpgroup is done; restage,

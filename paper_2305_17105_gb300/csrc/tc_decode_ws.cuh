@@ -327,16 +327,11 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_kernel(
       }
       out_activate(yv, M.out_act);
       if (tri) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          float s = yv[c] * wtap;
-          s += __shfl_xor_sync(0xffffffffu, s, 1);
-          s += __shfl_xor_sync(0xffffffffu, s, 2);
-          s += __shfl_xor_sync(0xffffffffu, s, 4);
-          yv[c] = s;
-        }
+        const int c = blend_taps(yv, wtap, row);
+        if (valid) store_pair(out, out_dtype, q * C, C, c, yv[0], yv[1]);
+      } else if (valid) {
+        store_texel(out, out_dtype, q, C, yv);
       }
-      if (valid && (!tri || (row & 7) == 0)) store_texel(out, out_dtype, q, C, yv);
       if (*abort_flag) break;
     }
   }
