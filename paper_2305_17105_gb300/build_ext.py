@@ -35,7 +35,9 @@ def _newer(target: str, deps) -> bool:
 def build(force: bool = False, verbose: bool = False, extra=()) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
-    sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+    # the longest units (the fused training step) first
+    sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")),
+                     key=lambda f: (not os.path.basename(f).startswith("tc_train"), f))
     headers = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         [os.path.join(ROOT, "include", "ntc.h")]
     objs, jobs = [], []

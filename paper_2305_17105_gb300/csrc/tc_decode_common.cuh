@@ -407,6 +407,7 @@ __device__ __forceinline__ void taps_of(int x, int y, float sx, float sy, int gw
 // Filled one tile ahead so the gathers overlap the previous tile's MMAs.
 struct Row {
   uint2 c0[4], c1[4];  // cells of the 4 taps of G0 / G1 (at most 8 bytes each)
+  uint32_t d0[4], d1[4];  // lattice form: bytes 8..11 of wider cells
   int frac;            // tap fractions in 1/16: fx0 | fy0 << 4 | fx1 << 8 | fy1 << 12
   float wtap;          // trilinear blend weight of this row
   int x, y, m;
@@ -856,6 +857,162 @@ __device__ __forceinline__ void generic_grid(const ntc_material& M, const MipTab
     }
 }
 
+// ---------------------------------------------------------------------------
+// Lattice form of the generic layout: packed grids of 2 or 4 bits whose taps
+// lie on the 1/16 lattice and whose bin widths are powers of two
+// (fast_layout_ok), in any cell size.  Channels stay in order, so the rows
+// equal the generic layout's, and every value is exact: both axes are blended
+// on the integer lattice, x in byte lanes (<= 240), y in the mantissas of
+// halves ((lerp - 256 off) Q / 256 has at most 11 significant bits).
+// Dequantising and blending in float, cell by cell, 10^6 queries of the
+// paper's profile 0.5 (G0 12 x 4 bits learned, G1 20 x 4 bits, three hidden
+// layers, C = 9) took 202 us; 88 now (with the row stores below and the fifth
+// pipeline).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void load_cells(const uint8_t* g, int cb, const int (&cell)[4],
+                                           uint2 (&c)[4], uint32_t (&d)[4]) {
+  if (cb == 8) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) c[t] = __ldg(reinterpret_cast<const uint2*>(g) + cell[t]);
+  } else if (cb == 16) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(g) + cell[t]);
+      c[t] = make_uint2(v.x, v.y);
+      d[t] = v.z;
+    }
+  } else if (cb == 4) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) c[t].x = __ldg(reinterpret_cast<const uint32_t*>(g) + cell[t]);
+  } else if (cb == 2) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) c[t].x = __ldg(reinterpret_cast<const unsigned short*>(g) + cell[t]);
+  } else {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) c[t].x = __ldg(g + cell[t]);
+  }
+}
+
+// Issue the eight cell loads of a row (invalid rows load nothing).
+__device__ __forceinline__ void gather_lattice(const Plan& P, const MipTab* tb, Row& r) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    r.c0[t] = r.c1[t] = make_uint2(0, 0);
+    r.d0[t] = r.d1[t] = 0;
+  }
+  r.frac = 0;
+  if (!r.valid) return;
+  const int x2 = 2 * r.x + 1, y2 = 2 * r.y + 1;
+  int cell[4], f0, f1;
+  taps16(x2, y2, tb->tk0[r.m], cell, f0);
+  load_cells(tb->grid0[r.m], P.cb0, cell, r.c0, r.d0);
+  taps16(x2, y2, tb->tk1[r.m], cell, f1);
+  load_cells(tb->grid1[r.m], P.cb1, cell, r.c1, r.d1);
+  r.frac = f0 | (f1 << 8);
+}
+
+// Word f of a cell.
+__device__ __forceinline__ uint32_t cell_word(const uint2& c, uint32_t d, int f) {
+  return f == 0 ? c.x : (f == 1 ? c.y : d);
+}
+
+// Channels 8 g .. 8 g + 7 of the four taps, bilinear.
+__device__ __forceinline__ uint4 lattice_group(const uint2 (&c)[4], const uint32_t (&d)[4], int bits,
+                                               int g, uint32_t wx0, uint32_t wx1, const YLerp& y) {
+  if (bits == 4) {
+    uint32_t e[4], o[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const uint32_t w = cell_word(c[t], d[t], g);
+      e[t] = w & 0x0F0F0F0Fu;         // channels 0 2 4 6
+      o[t] = (w >> 4) & 0x0F0F0F0Fu;  // channels 1 3 5 7
+    }
+    const uint32_t e0 = e[0] * wx0 + e[1] * wx1, e1 = e[2] * wx0 + e[3] * wx1;
+    const uint32_t o0 = o[0] * wx0 + o[1] * wx1, o1 = o[2] * wx0 + o[3] * wx1;
+    const uint32_t p0 = __byte_perm(e0, o0, 0x5140u), p1 = __byte_perm(e1, o1, 0x5140u);
+    const uint32_t q0 = __byte_perm(e0, o0, 0x7362u), q1 = __byte_perm(e1, o1, 0x7362u);
+    return make_uint4(ylerp(p0, p1, 0x4140u, y), ylerp(p0, p1, 0x4342u, y), ylerp(q0, q1, 0x4140u, y),
+                      ylerp(q0, q1, 0x4342u, y));
+  }
+  // 2 bits: the word's 16 channels in four registers, j holding channels
+  // j, 4 + j, 8 + j, 12 + j; the group's eight in bytes 2 (g & 1) and the next
+  uint32_t l0[4], l1[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    uint32_t v[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = (cell_word(c[t], d[t], g >> 1) >> (2 * j)) & 0x03030303u;
+    l0[j] = v[0] * wx0 + v[1] * wx1;
+    l1[j] = v[2] * wx0 + v[3] * wx1;
+  }
+  const uint32_t sel = (g & 1) ? 0x7362u : 0x5140u;
+  const uint32_t p0 = __byte_perm(l0[0], l0[1], sel), p1 = __byte_perm(l1[0], l1[1], sel);
+  const uint32_t q0 = __byte_perm(l0[2], l0[3], sel), q1 = __byte_perm(l1[2], l1[3], sel);
+  return make_uint4(ylerp(p0, p1, 0x4140u, y), ylerp(q0, q1, 0x4140u, y), ylerp(p0, p1, 0x4342u, y),
+                    ylerp(q0, q1, 0x4342u, y));
+}
+
+// Channels 8 g .. 8 g + 7 of one tap, dequantised: (1024 + k) Q - (1024 + off) Q.
+__device__ __forceinline__ uint4 lattice_tap(const uint2& c, uint32_t d, int bits, int g, __half2 q,
+                                             __half2 o) {
+  const uint32_t w = cell_word(c, d, bits == 4 ? g : g >> 1), kk = 0x64646464u;
+  auto dq = [&](uint32_t a, uint32_t sel) { return h2u(__hfma2(u2h(__byte_perm(a, kk, sel)), q, o)); };
+  if (bits == 4) {
+    const uint32_t e = w & 0x0F0F0F0Fu, od = (w >> 4) & 0x0F0F0F0Fu;
+    const uint32_t p = __byte_perm(e, od, 0x5140u), r = __byte_perm(e, od, 0x7362u);
+    return make_uint4(dq(p, 0x4140u), dq(p, 0x4342u), dq(r, 0x4140u), dq(r, 0x4342u));
+  }
+  const uint32_t sel = (g & 1) ? 0x7362u : 0x5140u;
+  const uint32_t p = __byte_perm(w & 0x03030303u, (w >> 2) & 0x03030303u, sel);
+  const uint32_t r = __byte_perm((w >> 4) & 0x03030303u, (w >> 6) & 0x03030303u, sel);
+  return make_uint4(dq(p, 0x4140u), dq(r, 0x4140u), dq(p, 0x4342u), dq(r, 0x4342u));
+}
+
+// Per-grid FP16 constants of the lattice form (off: the index of value zero).
+struct LatticeK {
+  __half2 s[2], s16[2], moff[2], q0, o0;
+  __device__ explicit LatticeK(const ntc_material& M) {
+    const float qq[2] = {M.q0, M.q1};
+    const int bits[2] = {M.bits0, M.bits1};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      s[k] = __float2half2_rn(qq[k] * (1.f / 256.f));
+      s16[k] = __float2half2_rn(qq[k] * (16.f / 256.f));
+      moff[k] = __float2half2_rn(-(float)((1 << (bits[k] - 1)) - 1) * qq[k]);
+    }
+    q0 = __float2half2_rn(M.q0);
+    o0 = __float2half2_rn(-(float)(1024 + (1 << (M.bits0 - 1)) - 1) * M.q0);
+  }
+};
+
+template <class S>
+__device__ __forceinline__ void build_lattice(const ntc_material& M, const Plan& P, const LatticeK& K,
+                                              const uint8_t* sm, const Row& r, const S& dst) {
+  if (P.learned) {
+    const int per = (M.c0 + 7) / 8;
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int g = 0; g < kGridPad / 8; ++g)
+        if (g < per) dst.put4(t * per + g, lattice_tap(r.c0[t], r.d0[t], M.bits0, g, K.q0, K.o0));
+  } else {
+    const uint32_t fx = r.frac & 15;
+    const YLerp y = ylerp_of((r.frac >> 4) & 15, K.s[0], K.s16[0], K.moff[0]);
+#pragma unroll
+    for (int g = 0; g < kGridPad / 8; ++g)
+      if (g < P.f0) dst.put4(g, lattice_group(r.c0, r.d0, M.bits0, g, 16 - fx, fx, y));
+  }
+  {
+    const uint32_t fx = (r.frac >> 8) & 15;
+    const YLerp y = ylerp_of((r.frac >> 12) & 15, K.s[1], K.s16[1], K.moff[1]);
+#pragma unroll
+    for (int g = 0; g < kGridPad / 8; ++g)
+      if (g < P.f1) dst.put4(P.f0 + g, lattice_group(r.c1, r.d1, M.bits1, g, 16 - fx, fx, y));
+  }
+  const MipTab* tb = reinterpret_cast<const MipTab*>(sm + P.tab);
+  pe_groups(P, sm, tb->lodh[r.m], r.x, r.y, dst);
+}
+
 template <bool F8, class S, bool VQ = true>
 __device__ __forceinline__ void build_generic(const ntc_material& M, const Plan& P,
                                               const uint8_t* sm, const Row& r, const S& dst,
@@ -1020,6 +1177,49 @@ __device__ __forceinline__ void store_texel_at(uint8_t* out, int mis, int out_dt
 __device__ __forceinline__ void store_texel(void* out, int out_dtype, int64_t q, int C,
                                             const float (&yv)[16]) {
   store_texel_at(static_cast<uint8_t*>(out), 0, out_dtype, q * C, C, yv);
+}
+
+// The first `rows` texels of a warp's 32 consecutive output rows, C values
+// each, from element e0 of `out` (e0 a multiple of 32 C): channel counts that
+// are not multiples of four leave no vector inside a row, but the warp's rows
+// are one contiguous block, so they pass through `st` (32 C floats of shared
+// memory) and leave as 16-byte vectors.  One store per value had every store
+// instruction touch 18 sectors (C = 9, FP16).
+__device__ __forceinline__ void store_rows(float* st, void* out, int out_dtype, int64_t e0, int rows,
+                                           int C, int lane, const float (&yv)[16]) {
+  float* mine = st + lane * C;
+#pragma unroll
+  for (int c = 0; c < 16; ++c)
+    if (c < C) mine[c] = yv[c];
+  __syncwarp();
+  const int cnt = rows * C;
+  const int per = out_dtype == NTC_DTYPE_F32 ? 4 : (out_dtype == NTC_DTYPE_F16 ? 8 : 16);
+  for (int i = lane * per; i < cnt; i += 32 * per) {
+    const float4* v4 = reinterpret_cast<const float4*>(st + i);
+    if (i + per <= cnt) {
+      uint4 w;
+      if (out_dtype == NTC_DTYPE_F32) {
+        w = *reinterpret_cast<const uint4*>(v4);
+      } else if (out_dtype == NTC_DTYPE_F16) {
+        const float4 a = v4[0], b = v4[1];
+        w = make_uint4(tc::pack_f16x2(a.x, a.y), tc::pack_f16x2(a.z, a.w), tc::pack_f16x2(b.x, b.y),
+                       tc::pack_f16x2(b.z, b.w));
+      } else {
+        const float4 a = v4[0], b = v4[1], c = v4[2], d = v4[3];
+        w = make_uint4(unorm8x4(a.x, a.y, a.z, a.w), unorm8x4(b.x, b.y, b.z, b.w),
+                       unorm8x4(c.x, c.y, c.z, c.w), unorm8x4(d.x, d.y, d.z, d.w));
+      }
+      const int eb = out_dtype == NTC_DTYPE_F32 ? 4 : (out_dtype == NTC_DTYPE_F16 ? 2 : 1);
+      *reinterpret_cast<uint4*>(static_cast<uint8_t*>(out) + (e0 + i) * eb) = w;
+    } else {
+      for (int j = i; j < cnt; ++j) {  // the call's last values
+        if (out_dtype == NTC_DTYPE_F32) static_cast<float*>(out)[e0 + j] = st[j];
+        else if (out_dtype == NTC_DTYPE_F16) static_cast<__half*>(out)[e0 + j] = __float2half_rn(st[j]);
+        else static_cast<uint8_t*>(out)[e0 + j] = (uint8_t)__float2uint_rn(__saturatef(st[j]) * 255.f);
+      }
+    }
+  }
+  __syncwarp();
 }
 
 // hardGELU (Sec. 4.4) as z * clamp(z/3 + 1/2, 0, 1): one saturating FMA and

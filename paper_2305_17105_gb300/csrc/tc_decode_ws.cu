@@ -1,6 +1,6 @@
-// Warp-specialised tensor-core decode (FP16), instantiated per fast-layout
-// class so that the per-row feature code has no runtime layout branches, and
-// its many-material form.
+// Warp-specialised tensor-core decode (FP16, one decode a query, rows of 4k
+// channels), instantiated per fast-layout class so that the per-row feature
+// code has no runtime layout branches, and its many-material form.
 #include "tc_decode_ws.cuh"
 
 namespace ntc {
@@ -42,7 +42,6 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_batched_kernel(
   __shared__ uint32_t tmem_base;
   __shared__ int wg_abort[kWsCompute];
   __shared__ int kint_s[kWsCompute];
-  __shared__ uint32_t desc_s[kWsCompute];
   __shared__ ntc_material mat_s[kWsCompute];
   constexpr bool FAST = CLS != 0;
   using Lay = FastLayout<(CLS > 0 ? CLS : 1)>;
@@ -76,7 +75,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_batched_kernel(
   const int per_tile = tri ? kRows / 8 : kRows;
   const int nm = B->n_materials;
   const int64_t total = B->total_tiles;
-  const int w = wg < kWsCompute ? wg : (warp & 3);
+  const int w = __shfl_sync(0xffffffffu, wg < kWsCompute ? wg : (warp & 3), 0);  // warp-uniform
   const int64_t nwgs = (int64_t)gridDim.x * kWsCompute, gw = (int64_t)blockIdx.x * kWsCompute + w;
   // tile indices fit 32 bits (ntc_batch_prepare refuses larger batches)
   const int t_begin = (int)(total * gw / nwgs), t_end = (int)(total * (gw + 1) / nwgs);
@@ -87,40 +86,50 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_batched_kernel(
 
   if (wg == kWsCompute) {
     // ---- issuer warp w ------------------------------------------------------
-    if (lane == 0) {
-      const uint32_t xa = tc::smem_u32(xtile);
-      const uint64_t cst = tc::smem_desc(tc::smem_u32(smem_raw + S.cst), 2048, 128);
-      uint32_t px = 0, ph = 0;
-      bool ok = true;
-      for (int tl = t_begin; tl < t_end; ++tl) {
-        if (!(ok = tc::mbar_wait(&bar_x[w], px, kWaitLimit))) break;
-        px ^= 1;
-        tc::fence_after_sync();
-        const uint64_t* d = reinterpret_cast<const uint64_t*>(
-            region + *reinterpret_cast<volatile uint32_t*>(&desc_s[w]));
-        const int k1 = *reinterpret_cast<volatile int*>(&kint_s[w]) / 16;
-        for (int s = 0; s < k1; ++s)
-          tc::mma_f16(tw, tc::smem_desc(xa + s * 4096, 2048, 128), d[s], id64, s > 0);
+    // (as in decode_ws_kernel: descriptors in registers, the elected lane of
+    // a converged warp issues)
+    constexpr uint32_t lbo = (kHidden / 8) * 128, lbo3 = (kN3 / 8) * 128;
+    const uint32_t xa = tc::desc_lo(tc::smem_u32(xtile), 2048);
+    const uint32_t cst = tc::desc_lo(tc::smem_u32(smem_raw + S.cst), 2048);
+    const uint32_t rg = tc::smem_u32(region);
+    auto dsc = [](uint32_t lo) { return tc::desc_of(lo, 128); };
+    auto wait_all = [](uint64_t* bar, uint32_t phase) {
+      return __all_sync(0xffffffffu, tc::mbar_wait(bar, phase, kWaitLimit)) != 0;
+    };
+    auto layer = [&](uint32_t d, uint32_t id, uint32_t b, uint32_t step, uint32_t bb, uint64_t* bar) {
+      if (!tc::elect_one()) return;
+#pragma unroll
+      for (int s = 0; s < kHidden / 16; ++s)
+        tc::mma_f16_ta(d, tw + kColH + 8 * s, dsc(b + s * step), id, s > 0);
+      tc::mma_f16(d, dsc(cst), dsc(bb), id, 1);
+      tc::mma_commit(bar);
+    };
+    uint32_t px = 0, ph = 0;
+    bool ok = true;
+    for (int tl = t_begin; tl < t_end; ++tl) {
+      if (!(ok = wait_all(&bar_x[w], px))) break;
+      px ^= 1;
+      tc::fence_after_sync();
+      // the region's tiles in Plan order: W1, W2, W3, the bias blocks
+      const int k = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&kint_s[w]), 0);
+      const uint32_t w1 = tc::desc_lo(rg, lbo), o2 = rg + kHidden * 2 * k, o3 = o2 + kHidden * kHidden * 2;
+      const uint32_t ob2 = o3 + kN3 * kHidden * 2, ob3 = ob2 + kHidden * 32;
+      if (tc::elect_one()) {
+        for (int s = 0; s < k / 16; ++s) tc::mma_f16(tw, dsc(xa + 256 * s), dsc(w1 + 128 * s), id64, s > 0);
         tc::mma_commit(&bar_d[w]);
-        if (!(ok = tc::mbar_wait(&bar_h[w], ph, kWaitLimit))) break;
-        ph ^= 1;
-        tc::fence_after_sync();
-        for (int s = 0; s < kHidden / 16; ++s)
-          tc::mma_f16_ta(tw, tw + kColH + 8 * s, d[kDescW2 + s], id64, s > 0);
-        tc::mma_f16(tw, cst, d[kDescW2 + 4], id64, 1);
-        tc::mma_commit(&bar_d[w]);
-        if (!(ok = tc::mbar_wait(&bar_h[w], ph, kWaitLimit))) break;
-        ph ^= 1;
-        tc::fence_after_sync();
-        for (int s = 0; s < kHidden / 16; ++s)
-          tc::mma_f16_ta(tw + kColD3, tw + kColH + 8 * s, d[kDescW3 + s], id16, s > 0);
-        tc::mma_f16(tw + kColD3, cst, d[kDescW3 + 4], id16, 1);
-        tc::mma_commit(&bar_o[w]);
       }
-      if (!ok) *reinterpret_cast<volatile int*>(&wg_abort[w]) = 1;
-      tc::mma_commit(&bar_fin[w]);
-      if (!tc::mbar_wait(&bar_fin[w], 0, kWaitLimit)) *reinterpret_cast<volatile int*>(&wg_abort[w]) = 1;
+      if (!(ok = wait_all(&bar_h[w], ph))) break;
+      ph ^= 1;
+      tc::fence_after_sync();
+      layer(tw, id64, tc::desc_lo(o2, lbo), 128, tc::desc_lo(ob2, lbo), &bar_d[w]);
+      if (!(ok = wait_all(&bar_h[w], ph))) break;
+      ph ^= 1;
+      tc::fence_after_sync();
+      layer(tw + kColD3, id16, tc::desc_lo(o3, lbo3), 32, tc::desc_lo(ob3, lbo3), &bar_o[w]);
     }
+    if (!ok) *reinterpret_cast<volatile int*>(&wg_abort[w]) = 1;
+    if (tc::elect_one()) tc::mma_commit(&bar_fin[w]);
+    if (!tc::mbar_wait(&bar_fin[w], 0, kWaitLimit)) *reinterpret_cast<volatile int*>(&wg_abort[w]) = 1;
   } else {
     // ---- compute warpgroup w -------------------------------------------------
     const uint32_t lq = (uint32_t)((warp & 3) * 32) << 16;
@@ -154,10 +163,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) decode_ws_batched_kernel(
       m_C = M.channels;
       stage_shared<false>(M, P, region, row, kRows);
       zero_tail_groups<false>(P, xs);
-      if (row == 0) {
-        kint_s[w] = P.k_int;
-        desc_s[w] = P.desc;
-      }
+      if (row == 0) kint_s[w] = P.k_int;
       m_t0 = (int)B->tile_start[id];
       m_t1 = (int)B->tile_start[id + 1];
       m_q0 = B->q_off[id];
@@ -340,37 +346,11 @@ cudaError_t launch_decode_ws_batched(const BatchHeader* dev, int64_t total_tiles
 
 cudaError_t launch_decode_ws(const ntc_material& m, const float* uvl, int64_t n, void* out,
                              int out_dtype, int filter, uint64_t jkey, cudaStream_t s, bool fast) {
-  if (m.hidden_layers == 3) {  // a third hidden layer: the paper's profiles, else run time
-    if (!fast) return launch_ws<0, false, true>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    const Plan P(m, false, true);
-    const int cls = P.vq ? -1 : (P.learned ? 11 : 1) + 3 * grid_class(m.c0, P.cb0) +
-                                    grid_class(m.c1, P.cb1);
-    if (cls == 16) return launch_ws<16, false, true>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    if (cls == 18) return launch_ws<18, false, true>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    return launch_ws<-1, false, true>(m, uvl, n, out, out_dtype, filter, jkey, s);
-  }
-  if (!fast) return launch_ws<0, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-  const Plan P(m, false, true);
-  if (P.vq) return launch_ws<-1, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-  if (P.learned) {
-    // the paper's profiles 0.5 and 2.25 (4-bit G0 of 12 / 16 channels, G1 of
-    // 16 / 12) as compile-time classes, other learned layouts at run time
-    switch (11 + 3 * grid_class(m.c0, P.cb0) + grid_class(m.c1, P.cb1)) {
-      case 16: return launch_ws<16, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-      case 18: return launch_ws<18, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-      default: return launch_ws<-1, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    }
-  }
-  switch (1 + 3 * grid_class(m.c0, P.cb0) + grid_class(m.c1, P.cb1)) {
-    case 1: return launch_ws<1, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    case 2: return launch_ws<2, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    case 3: return launch_ws<3, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    case 4: return launch_ws<4, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    case 5: return launch_ws<5, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    case 6: return launch_ws<6, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    case 7: return launch_ws<7, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    case 8: return launch_ws<8, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
-    default: return launch_ws<9, false>(m, uvl, n, out, out_dtype, filter, jkey, s);
+  switch (ws_mode(m, false, fast, filter, out_dtype)) {
+    case kWsStoch: return launch_decode_ws_stoch(m, uvl, n, out, out_dtype, filter, jkey, s, fast);
+    case kWsTri: return launch_decode_ws_tri(m, uvl, n, out, out_dtype, filter, jkey, s, fast);
+    case kWsRows: return launch_decode_ws_rows(m, uvl, n, out, out_dtype, filter, jkey, s, fast);
+    default: return dispatch_f16<kWsPlain>(m, uvl, n, out, out_dtype, filter, jkey, s, fast);
   }
 }
 

@@ -43,6 +43,25 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;                // base offset 0, relative LBO mode, layout type 0 (no swizzle)
 }
 
+// One lane of a converged warp, the same one every time.  tcgen05.mma takes
+// its operands from uniform registers: inside `if (elect_one())`, with
+// warp-uniform operands, a chain with A in TMEM advances 43 cycles a step
+// (N = 64); issued under a divergent `lane == 0`, 95.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
+// The two words of a descriptor: the low one holds the start address and the
+// leading offset, so stepping along K adds (byte step / 16) to it.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo) {
+  return ((saddr & 0x3FFFF) >> 4) | (((lbo & 0x3FFFF) >> 4) << 16);
+}
+__device__ __forceinline__ uint64_t desc_of(uint32_t lo, uint32_t sbo) {
+  return (uint64_t)lo | (uint64_t)(((sbo & 0x3FFFF) >> 4) | (1u << 14)) << 32;
+}
+
 // Instruction descriptor: D = F32, A/B type code 0 (F16 for kind::f16, E4M3
 // for kind::f8f6f4), both K-major, M x N.
 __host__ __device__ constexpr uint32_t idesc(int M, int N) {
@@ -142,6 +161,18 @@ __device__ __forceinline__ void tmem_st_wait() {
   asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
 }
 
+// This warpgroup's registers per thread: give some back to, or take some from,
+// the block's pool (its threads times the registers it was launched with).
+// `reg_inc` waits until the pool holds enough.
+template <int N>
+__device__ __forceinline__ void reg_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void reg_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(N));
+}
+
 // Arrive on an mbarrier once every previously issued MMA of this thread has
 // completed.
 __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
@@ -209,6 +240,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
       : "r"(taddr));
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");

@@ -62,3 +62,30 @@ def test_trilinear_rows(precision, channels):
         got = to_np(ntc.ntc_decode(mat, _uvl(q), out_dtype=dtype, filter=ntc.FILTER_TRILINEAR))
         half = 5e-4 if dtype == torch.float16 else 0.0
         assert np.abs(got - md.decode_trilinear(q)).max() <= tol + half
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16, torch.uint8])
+@pytest.mark.parametrize("channels", [8, 9, 13, 15])
+@pytest.mark.parametrize("precision", ["f16", "f8"])
+def test_rows_through_shared_memory(dtype, channels, precision):
+    """A call whose rows pass through shared memory against one of 16 channels
+    with the same first weights, stored row by row: the same values, nothing
+    written past the last row (a tile boundary, a warp's and a ragged end)."""
+    case = make_case(seed=151, width=64, height=64, channels=channels, c0=12, c1=12, k_in=64)
+    mat, md = device_material(case, precision=ntc.PREC_F16)
+    pad = lambda t: torch.cat([t, torch.zeros(16 - channels, *t.shape[1:], dtype=t.dtype, device=DEV)])
+    full = mat.with_(channels=16, weights=mat.weights[:2] + [pad(mat.weights[2])],
+                     biases=mat.biases[:2] + [pad(mat.biases[2])])
+    if precision == "f8":
+        scale = torch.tensor([2.0 ** -9, 2.0 ** -9, 2.0 ** -9, 2.0 ** -8, 2.0 ** -7, 2.0 ** -6],
+                             device=DEV)
+        e4 = lambda t: (t.float() * 512).clamp(-448, 448).to(torch.float8_e4m3fn).view(torch.uint8)
+        mat = mat.with_(weights=[e4(w) for w in mat.weights], precision=ntc.PREC_F8, scale=scale)
+        full = full.with_(weights=[e4(w) for w in full.weights], precision=ntc.PREC_F8, scale=scale)
+    for n in (1, 31, 33, 128, 161, 5 * 128 * 2 + 77):
+        q = _uvl(gen.random_queries(n, md.mips, seed=4151))
+        out = torch.full((n * channels + 64,), 7, dtype=dtype, device=DEV)
+        got = ntc.ntc_decode(mat, q, out=out)[:n * channels].view(n, channels)
+        assert torch.equal(got, ntc.ntc_decode(full, q, out_dtype=dtype)[:, :channels]), n
+        assert bool((out[n * channels:] == 7).all())
+    assert ntc.ntc_device_status() == ntc.OK
