@@ -1,10 +1,17 @@
 // Tensor-core (tcgen05) fused forward + L2 loss + backward of the NTC
 // optimisation step (Sec. 4.2, 4.5, 5.1), FP16 operands, FP32 accumulation.
 //
-// One persistent CTA per SM runs NWG warpgroup pipelines (3, 2 or 1: the most
-// whose tiles fit in shared memory); a warpgroup owns a stream of tiles of 128
-// training texels (one per thread = one row = one TMEM lane).  Per tile, with
-// every activation kept on chip:
+// One persistent CTA per SM runs NWG pipelines (3, 2 or 1: the most whose
+// tiles fit in shared memory); a pipeline of 256 threads owns a stream of
+// tiles of 128 training texels (one row = one TMEM lane each).  Two threads
+// share a row: half 0 gathers G0, half 1 G1 and the encoding; in every
+// epilogue each takes one half of the columns, in the scatter one half of the
+// warp's texels.  The step is bound by the latency of a tile's serial chain
+// (issue slots a fifth used).  With one thread a row and the MMAs issued by a
+// divergent thread a tile alone took 12.6 us, now 8.9; a step of 2^18 texels
+// of a 2048^2 x 12 material 176 -> 160 us, of eight crops on the paper's
+// decoder 353 -> 268 us.
+// Per tile, with every activation kept on chip:
 //   forward   X -> Z1 = X W1^T (+b1) -> H1 = act(Z1) -> Z2 (+b2) -> H2 -> Z3 (+b3)
 //             -> y = out(Z3), loss, dZ3 = 2 (y - t) out'(Z3); with a third
 //             hidden layer H2 -> Zh (+bh) -> H3 feeds the output layer, and
@@ -58,7 +65,8 @@ namespace {
 
 constexpr int kRows = 128;
 constexpr int kN3 = 16;
-constexpr int kMaxNWG = 3;              // warpgroup pipelines per CTA (at most)
+constexpr int kMaxNWG = 3;              // pipelines per CTA (at most)
+constexpr int kPipe = 2 * kRows;        // threads of a pipeline: two per row
 constexpr uint32_t kCols = 512;         // TMEM columns of the CTA
 constexpr uint32_t kGroup = 2048;       // bytes per 8-unit group of a 128-row tile
 constexpr uint32_t kWaitLimit = 1u << 18;  // suspended tries: ms to seconds
@@ -394,54 +402,15 @@ __device__ __forceinline__ uint32_t xlo_group(const TPlan& P, int g) {
   return g < 8 ? P.H1 + (uint32_t)g * kGroup : P.H2 + (uint32_t)(g - 8) * kGroup;
 }
 
-// 64 values of a TMEM row (starting at column `col`) -> f(v) -> 8 FP16
-// chunks of a tile.
-template <class F>
-__device__ __forceinline__ void row64_to_tile(uint32_t taddr, uint8_t* tile, int row, F f) {
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    float a[16], b[16];
-    tc::tmem_ld16(taddr + 32 * half, a);
-    tc::tmem_ld16(taddr + 32 * half + 16, b);
-    tc::tmem_ld_wait();
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      float v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int i = 8 * g + e;
-        v[e] = f(32 * half + i, i < 16 ? a[i] : b[i - 16]);
-      }
-      put_chunk(tile, row, 4 * half + g, v);
-    }
-  }
-}
-
-// One tile's own row of an FP16 tile, unpacked (8 groups = 64 values).
-__device__ __forceinline__ void tile_row64(const uint8_t* tile, int row, __half2 (&h)[32]) {
-#pragma unroll
-  for (int g = 0; g < 8; ++g) {
-    const uint4 w = *reinterpret_cast<const uint4*>(tile + tc::canon_chunk(row, g, kRows));
-    const uint32_t u[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      union { uint32_t u; __half2 h; } c;
-      c.u = u[j];
-      h[4 * g + j] = c.h;
-    }
-  }
-}
-
-__device__ __forceinline__ float half_of(const __half2 (&h)[32], int i) {
-  return (i & 1) ? __high2float(h[i >> 1]) : __low2float(h[i >> 1]);
-}
 
 __device__ __forceinline__ void issue_kmajor(uint32_t d, uint32_t a, uint32_t a_lbo, uint32_t b,
                                              uint32_t b_lbo, int ksteps, uint32_t id,
                                              uint32_t acc0) {
+  const uint32_t al = tc::desc_lo(a, a_lbo), bl = tc::desc_lo(b, b_lbo);
+#pragma unroll 4
   for (int s = 0; s < ksteps; ++s)
-    tc::mma_f16(d, tc::smem_desc(a + 2 * s * a_lbo, a_lbo, 128),
-                tc::smem_desc(b + 2 * s * b_lbo, b_lbo, 128), id, (s > 0) | acc0);
+    tc::mma_f16(d, tc::desc_of(al + s * (a_lbo / 8), 128), tc::desc_of(bl + s * (b_lbo / 8), 128), id,
+                (s > 0) | acc0);
 }
 
 // MN-major operands with K = the 128 texels of the tile: 8 K-steps of 16
@@ -451,9 +420,10 @@ __device__ __forceinline__ void issue_kmajor(uint32_t d, uint32_t a, uint32_t a_
 // 8-texel groups, 128 bytes apart), as in the K-major case.
 __device__ __forceinline__ void issue_mnmajor(uint32_t d, uint32_t a, uint32_t b, uint32_t id,
                                               uint32_t acc0) {
+  const uint32_t al = tc::desc_lo(a, 128), bl = tc::desc_lo(b, 128);
+#pragma unroll
   for (int s = 0; s < kRows / 16; ++s)
-    tc::mma_f16(d, tc::smem_desc(a + 256 * s, 128, kGroup), tc::smem_desc(b + 256 * s, 128, kGroup),
-                id, (s > 0) | acc0);
+    tc::mma_f16(d, tc::desc_of(al + 16 * s, kGroup), tc::desc_of(bl + 16 * s, kGroup), id, (s > 0) | acc0);
 }
 
 // 32-byte read-only global load (sm_100+), 32-byte aligned address.
@@ -463,48 +433,38 @@ __device__ __forceinline__ void ld_nc_v8(const float* p, float4& a, float4& b) {
       : "l"(p));
 }
 
-// Bilinear sample of one FP32 grid of 4k <= 16 channels with 16-byte loads,
-// all taps' loads issued before the interpolation (same FMA order as
-// sample_grid, so the same values).
-// `base` (nullable) replaces the level's grid pointer (the trainer's noisy
-// copy of the same layout).
-__device__ __forceinline__ void sample_grid_f32x4(const ntc_material& M, int j, int k, int x, int y,
-                                                  int wm, int hm, GridSample& gs,
-                                                  const float* base = nullptr) {
-  const ntc_level& L = M.lv[j];
-  const int gw = k ? L.g1_w : L.g0_w, gh = k ? L.g1_h : L.g0_h;
-  const int c4 = (k ? M.c1 : M.c0) >> 2;
-  const Taps t = bilinear_taps(x, y, wm, hm, gw, gh);
-  const float4* g = static_cast<const float4*>(base ? static_cast<const void*>(base) : (k ? L.grid1 : L.grid0));
-  float4 v[4][kFastGridCh / 4];
-  if ((c4 == 2 || c4 == 4) && (reinterpret_cast<uintptr_t>(g) & 31) == 0) {
-    // 32-byte loads: one L1 wavefront brings 8 channels
+// Channels 8 g .. 8 g + 7 (those below c; the others are zero) of the bilinear
+// sample of one FP32 grid of c = 4k <= 16 channels at `base`: all taps' loads
+// issued before the interpolation (same FMA order as sample_grid, so the same
+// values); 32-byte loads where every group is whole and aligned (one L1
+// wavefront brings 8 channels).
+__device__ __forceinline__ void sample_group_f32(const float* base, int c, const Taps& t, int g,
+                                                 float (&v)[8]) {
+  const bool wide = (c & 7) == 0 && (reinterpret_cast<uintptr_t>(base) & 31) == 0;
+  float4 a[4], b[4];
 #pragma unroll
-    for (int tp = 0; tp < 4; ++tp)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (2 * h < c4) ld_nc_v8(reinterpret_cast<const float*>(g + (size_t)t.cell[tp] * c4 + 2 * h),
-                                 v[tp][2 * h], v[tp][2 * h + 1]);
-        else v[tp][2 * h] = v[tp][2 * h + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-  } else {
-#pragma unroll
-    for (int tp = 0; tp < 4; ++tp)
-#pragma unroll
-      for (int q = 0; q < kFastGridCh / 4; ++q)
-        v[tp][q] = q < c4 ? __ldg(g + (size_t)t.cell[tp] * c4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int tp = 0; tp < 4; ++tp) {
+    const float* q = base + (size_t)t.cell[tp] * c + 8 * g;
+    if (wide) {
+      ld_nc_v8(q, a[tp], b[tp]);
+    } else {
+      a[tp] = __ldg(reinterpret_cast<const float4*>(q));
+      b[tp] = 8 * g + 4 < c ? __ldg(reinterpret_cast<const float4*>(q) + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
 #pragma unroll
-  for (int ch = 0; ch < kGridPad; ++ch) gs.acc[ch] = 0.f;
+  for (int e = 0; e < 8; ++e) v[e] = 0.f;
 #pragma unroll
-  for (int tp = 0; tp < 4; ++tp)
-#pragma unroll
-    for (int q = 0; q < kFastGridCh / 4; ++q) {
-      gs.acc[4 * q] = fmaf(t.w[tp], v[tp][q].x, gs.acc[4 * q]);
-      gs.acc[4 * q + 1] = fmaf(t.w[tp], v[tp][q].y, gs.acc[4 * q + 1]);
-      gs.acc[4 * q + 2] = fmaf(t.w[tp], v[tp][q].z, gs.acc[4 * q + 2]);
-      gs.acc[4 * q + 3] = fmaf(t.w[tp], v[tp][q].w, gs.acc[4 * q + 3]);
-    }
+  for (int tp = 0; tp < 4; ++tp) {
+    v[0] = fmaf(t.w[tp], a[tp].x, v[0]);
+    v[1] = fmaf(t.w[tp], a[tp].y, v[1]);
+    v[2] = fmaf(t.w[tp], a[tp].z, v[2]);
+    v[3] = fmaf(t.w[tp], a[tp].w, v[3]);
+    v[4] = fmaf(t.w[tp], b[tp].x, v[4]);
+    v[5] = fmaf(t.w[tp], b[tp].y, v[5]);
+    v[6] = fmaf(t.w[tp], b[tp].z, v[6]);
+    v[7] = fmaf(t.w[tp], b[tp].w, v[7]);
+  }
 }
 
 // K-major A, MN-major B: a forward weight tile [out][in] (K-major, `R` rows
@@ -512,19 +472,19 @@ __device__ __forceinline__ void sample_grid_f32x4(const ntc_material& M, int j, 
 // along K (8 outputs) and (R / 8) * 128 bytes along N.
 __device__ __forceinline__ void issue_kmn(uint32_t d, uint32_t a, uint32_t a_lbo, uint32_t b,
                                           uint32_t b_sbo, int ksteps, uint32_t id) {
+  const uint32_t al = tc::desc_lo(a, a_lbo), bl = tc::desc_lo(b, 128);
+#pragma unroll 4
   for (int s = 0; s < ksteps; ++s)
-    tc::mma_f16(d, tc::smem_desc(a + 2 * s * a_lbo, a_lbo, 128),
-                tc::smem_desc(b + 256 * s, 128, b_sbo), id, s > 0);
+    tc::mma_f16(d, tc::desc_of(al + s * (a_lbo / 8), 128), tc::desc_of(bl + 16 * s, b_sbo), id, s > 0);
 }
 
-// Forward epilogue of a hidden layer: H = act(Z) into `htile` (FP16 heads;
-// with `ltile` the FP16 tails go there); hardGELU also writes act'(Z) into
-// `gtile`.
+// Forward epilogue of a hidden layer, columns 32 half .. +31 of a row: H =
+// act(Z) into `htile` (FP16 heads; with `ltile` the FP16 tails go there);
+// hardGELU also writes act'(Z) into `gtile`.
 template <int ACT>
 __device__ __forceinline__ void hidden_forward(uint32_t taddr, uint8_t* htile, uint8_t* gtile,
-                                               uint8_t* ltile, int row) {
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
+                                               uint8_t* ltile, int row, int half) {
+  {
     float a[16], b[16];
     tc::tmem_ld16(taddr + 32 * half, a);
     tc::tmem_ld16(taddr + 32 * half + 16, b);
@@ -579,9 +539,8 @@ __device__ __forceinline__ void put_x8(uint8_t* W, const TPlan& P, int row, int 
 template <int ACT>
 __device__ __forceinline__ void hidden_forward_f8(uint32_t taddr, float s_in, const float* bias,
                                                   float inv, uint8_t* h16, uint8_t* h8,
-                                                  uint8_t* gtile, int row, float& amax) {
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
+                                                  uint8_t* gtile, int row, int half, float& amax) {
+  {
     float a[16], b[16];
     tc::tmem_ld16(taddr + 32 * half, a);
     tc::tmem_ld16(taddr + 32 * half + 16, b);
@@ -620,31 +579,48 @@ __device__ __forceinline__ void hidden_forward_f8(uint32_t taddr, float s_in, co
 
 __device__ __forceinline__ void issue_kmajor_f8(uint32_t d, uint32_t a, uint32_t a_lbo, uint32_t b,
                                                 uint32_t b_lbo, int ksteps, uint32_t id) {
+  const uint32_t al = tc::desc_lo(a, a_lbo), bl = tc::desc_lo(b, b_lbo);
+#pragma unroll 4
   for (int s = 0; s < ksteps; ++s)
-    tc::mma_f8(d, tc::smem_desc(a + 2 * s * a_lbo, a_lbo, 128),
-               tc::smem_desc(b + 2 * s * b_lbo, b_lbo, 128), id, s > 0);
+    tc::mma_f8(d, tc::desc_of(al + s * (a_lbo / 8), 128), tc::desc_of(bl + s * (b_lbo / 8), 128), id, s > 0);
 }
 
-// Backward epilogue: dZ = dH * act'(Z) over the layer's H tile (this row is
-// read before it is overwritten): ReLU takes act' from the sign of H,
+// Backward epilogue, columns 32 half .. +31 of a row: dZ = dH * act'(Z) over
+// the layer's H tile (each chunk is read before it is overwritten): ReLU takes act' from the sign of H,
 // hardGELU from the forward's G tile.
 // FP8 form: the accumulator is dZ_next W8 (E4M3 weight values), scaled by
 // the layer's weight scale `sc`; a ReLU unit's mask is any nonzero bit
 // pattern of H (its -0 marks a positive Z whose value rounded to zero).
 template <int ACT, bool F8>
 __device__ __forceinline__ void hidden_backward(uint32_t taddr, const uint8_t* gtile,
-                                                uint8_t* htile, int row, float sc = 1.f) {
-  __half2 h[32];
-  tile_row64(ACT == NTC_ACT_HARDGELU ? gtile : htile, row, h);
-  row64_to_tile(taddr, htile, row, [&](int q, float g) {
-    if (F8) g *= sc;
-    if (ACT == NTC_ACT_HARDGELU) return g * half_of(h, q);
-    if (F8) {
-      const __half hv = (q & 1) ? __high2half(h[q >> 1]) : __low2half(h[q >> 1]);
-      return __half_as_ushort(hv) != 0 ? g : 0.f;
+                                                uint8_t* htile, int row, int half, float sc = 1.f) {
+  const uint8_t* src = ACT == NTC_ACT_HARDGELU ? gtile : htile;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    float a[16];
+    tc::tmem_ld16(taddr + 32 * half + 16 * q, a);
+    uint4 hw[2];
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+      hw[g] = *reinterpret_cast<const uint4*>(src + tc::canon_chunk(row, 4 * half + 2 * q + g, kRows));
+    tc::tmem_ld_wait();
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const uint32_t u[4] = {hw[g].x, hw[g].y, hw[g].z, hw[g].w};
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint32_t hb = (u[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
+        const float h = __half2float(__ushort_as_half((unsigned short)hb));
+        float d = a[8 * g + e];
+        if (F8) d *= sc;
+        if (ACT == NTC_ACT_HARDGELU) v[e] = d * h;
+        else if (F8) v[e] = hb != 0u ? d : 0.f;
+        else v[e] = h > 0.f ? d : 0.f;
+      }
+      put_chunk(htile, row, 4 * half + 2 * q + g, v);
     }
-    return half_of(h, q) > 0.f ? g : 0.f;
-  });
+  }
 }
 
 // X slot s of a row: FP16 head into X, FP16 tail into X's tail groups.
@@ -676,9 +652,12 @@ __device__ __forceinline__ void put_x(uint8_t* W, const TPlan& P, int row, int g
 // Learned interpolation of G0 (Sec. 4.3.1): the c0 values of the four
 // bilinear-footprint cells at slots tap * c0 + ch, zeros up to the group
 // boundary.  FP32 grid values (plus this step's noise when asked).
+// HALF 0 writes taps 0 to 2, half 1 tap 3 and the zeros.
+template <int HALF>
 __device__ __forceinline__ void learned_g0(const ntc_material& M, const TPlan& P, int j, int x,
                                            int y, int wm, int hm, bool valid, bool noise,
                                            uint64_t nkey, uint8_t* W, int row) {
+  constexpr int T0 = HALF ? 3 : 0, T1 = HALF ? 4 : 3;
   const ntc_level& L = M.lv[j];
   const Taps t = bilinear_taps(x, y, wm, hm, L.g0_w, L.g0_h);
   const int c = M.c0;
@@ -686,25 +665,26 @@ __device__ __forceinline__ void learned_g0(const ntc_material& M, const TPlan& P
     const float* g = static_cast<const float*>(L.grid0);
     float4 v[4][kFastGridCh / 4];
 #pragma unroll
-    for (int tp = 0; tp < 4; ++tp)
+    for (int tp = T0; tp < T1; ++tp)
 #pragma unroll
       for (int q = 0; q < kFastGridCh / 4; ++q)
         v[tp][q] = (valid && 4 * q < c)
                        ? __ldg(reinterpret_cast<const float4*>(g + (size_t)t.cell[tp] * c) + q)
                        : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int tp = 0; tp < 4; ++tp)
+    for (int tp = T0; tp < T1; ++tp)
 #pragma unroll
       for (int q = 0; q < kFastGridCh / 4; ++q)
         if (4 * q < c) put_half4(W, P, row, tp * c + 4 * q, v[tp][q]);
   } else {
 #pragma unroll
-    for (int tp = 0; tp < 4; ++tp)
+    for (int tp = T0; tp < T1; ++tp)
       for (int ch = 0; ch < c; ++ch)
         put_half(W, P, row, tp * c + ch,
                  valid ? grid_value<true>(M, j, 0, t.cell[tp], ch, noise, nkey) : 0.f);
   }
-  for (int s = P.w0; s < 8 * P.f0; ++s) put_half(W, P, row, s, 0.f);
+  if (HALF)
+    for (int s = P.w0; s < 8 * P.f0; ++s) put_half(W, P, row, s, 0.f);
 }
 
 // Scatter-add of `d` (c values) into grid cell rows through four taps,
@@ -731,7 +711,7 @@ __device__ __forceinline__ void scatter_taps(float* g, int c, const Taps& t, con
 }
 
 // One lane's part of the coalesced grid scatter: slot `slot` (grid, tap) and
-// channels 4q .. 4q+3 of each of the warp's 32 texels, whose cell addresses
+// channels 4q .. 4q+3 of 16 texels, whose cell addresses
 // and weights sit at meta + t * kScatMeta and whose dX values at
 // dx + t * dx_stride.  MERGE: consecutive texels that share the cell are
 // summed in registers and reduced once per run (coherent texels: crops or
@@ -742,7 +722,7 @@ __device__ __forceinline__ void scatter_lane(const uint8_t* meta, const float* d
   float* run = nullptr;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-  for (int t = 0; t < 32; ++t) {
+  for (int t = 0; t < 16; ++t) {
     float* const ga = *reinterpret_cast<float* const*>(meta + t * kScatMeta + 8 * slot);
     if (MERGE) {
       if (ga != run) {
@@ -767,10 +747,11 @@ __device__ __forceinline__ void scatter_lane(const uint8_t* meta, const float* d
   if (MERGE && run) atomicAdd(reinterpret_cast<float4*>(run) + q, acc);
 }
 
-__device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t& phase, int bar_id) {
-  const bool ok = tc::mbar_wait(bar, phase, kWaitLimit);
+// Wait for the pipeline's MMAs; after a wait that ran out (`bad`) no further
+// one is tried, and the pipeline leaves at the end of the tile.
+__device__ __forceinline__ void wait_phase(uint64_t* bar, uint32_t& phase, bool& bad) {
+  if (!bad) bad = !tc::mbar_wait(bar, phase, kWaitLimit);
   phase ^= 1;
-  return !tc::bar_or(bar_id, kRows, !ok);
 }
 
 // BATCHED: the CTA takes an even share of the batch's tile list (ordered by
@@ -780,7 +761,7 @@ __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t& phase, int b
 // accumulators into that material's gradient.  Otherwise one material (M0,
 // A0) whose tiles the CTAs take in turn, NWG at a time.
 template <int ACT, bool LEARNED, int NWG, bool BATCHED, bool F8>
-__global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_material M0,
+__global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_material M0,
                                                                   const BwdArgs A0,
                                                                   const TrainBatchDev* hb,
                                                                   int k_lay, int dx_lay,
@@ -789,13 +770,17 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
   __shared__ uint64_t mbar[NWG], fin[NWG];
   __shared__ uint32_t tmem_base;
   __shared__ int abort_any;
-  __shared__ float red[NWG * 4];
+  __shared__ float red[NWG * 8];
   __shared__ uint32_t dout_max;  // bits of the CTA's largest |dout| (dout mode)
   // the current material and step arguments of a batched launch
   __shared__ __align__(16) uint8_t seg_buf[BATCHED ? sizeof(ntc_material) + sizeof(BwdArgs) : 16];
   uint8_t* sm = smem_raw;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int wg = tid / kRows, row = tid % kRows;
+  // pipeline and warp in it (warp-uniform for the MMAs' operands); row and
+  // which of its two threads
+  const int wg = __shfl_sync(0xffffffffu, tid / kPipe, 0);
+  const int pw = __shfl_sync(0xffffffffu, (tid % kPipe) >> 5, 0);
+  const int row = tid % kRows, hf = (tid / kRows) & 1;
   const int bar_id = 1 + wg;
   const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
   const ntc_material& M = BATCHED ? *reinterpret_cast<const ntc_material*>(seg_buf) : M0;
@@ -837,7 +822,7 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
       const uint32_t* src_a = reinterpret_cast<const uint32_t*>(&hb->args[seg]);
       uint32_t* dst = reinterpret_cast<uint32_t*>(seg_buf);
       constexpr int nm = sizeof(ntc_material) / 4, na = sizeof(BwdArgs) / 4;
-      for (int i = tid; i < nm + na; i += kRows * NWG) dst[i] = i < nm ? src_m[i] : src_a[i - nm];
+      for (int i = tid; i < nm + na; i += kPipe * NWG) dst[i] = i < nm ? src_m[i] : src_a[i - nm];
     }
     __syncthreads();
     t_lo = (c_begin > t0 ? c_begin : t0) - t0 + wg;
@@ -866,9 +851,9 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  // the shared weight-gradient accumulators start at zero (warpgroup 0 holds
+  // the shared weight-gradient accumulators start at zero (four warps hold
   // every lane; every MMA into them accumulates)
-  if (wg == 0) {
+  if (tid < kRows) {
     const uint32_t z[16] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (uint32_t c = P.colW1; c < P.cols; c += 16) tc::tmem_st16(tmem_base + c + lane, z);
     tc::tmem_st_wait();
@@ -879,7 +864,7 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
     for (int64_t tl = t_lo; tl < t_hi; tl += t_step) {
       const int64_t i = tl * kRows + row;
       if (i < A.n)
-        for (int c = 0; c < C; ++c) mx = fmaxf(mx, fabsf(A.dout[i * C + c]));
+        for (int c = hf; c < C; c += 2) mx = fmaxf(mx, fabsf(A.dout[i * C + c]));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -928,7 +913,7 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
   const bool noise_on = A.noise != 0 && !use_copy;
   const uint64_t skey = rng_key(A.sample_seed, sampler_stream(step));
   float loss_acc = 0.f;
-  bool aborted = false;
+  bool bad = false;
 
   for (int64_t tl = t_lo; tl < t_hi; tl += t_step) {
     const int64_t i = tl * kRows + row;
@@ -939,46 +924,66 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
       if (A.uvl) query_texel(M, A.uvl[3 * i], A.uvl[3 * i + 1], A.uvl[3 * i + 2], x, y, m);
       else sample_train_texel(A.crops != 0, skey, i, M.width, M.height, M.mips, x, y, m);
     }
-    // loss mode: the texel's C <= 16 target bytes, loaded here and parked in
-    // the (free) DZ3 tile once the features are built, so their latency
-    // hides behind the gathers; the loss reads them back
-    uint32_t tw[4] = {0u, 0u, 0u, 0u};
+    // loss mode: this half's 8 target bytes of the texel (channels 8 hf ..),
+    // loaded here so that their latency hides behind the gathers
+    uint32_t tw[2] = {0u, 0u};
     if (A.target && valid) {
-      const uint8_t* trow = A.target + A.tgt_off[m] + ((int64_t)y * tb->wm[m] + x) * C;
+      const uint8_t* trow = A.target + A.tgt_off[m] + ((int64_t)y * tb->wm[m] + x) * C + 8 * hf;
       if ((C & 3) == 0) {
         // whole 4-byte words of the u8 row (row offsets are multiples of 4)
 #pragma unroll
-        for (int c4 = 0; c4 < kN3 / 4; ++c4)
-          if (4 * c4 < C) tw[c4] = __ldg(reinterpret_cast<const uint32_t*>(trow) + c4);
+        for (int c4 = 0; c4 < 2; ++c4)
+          if (8 * hf + 4 * c4 < C) tw[c4] = __ldg(reinterpret_cast<const uint32_t*>(trow) + c4);
       } else {
 #pragma unroll
-        for (int c = 0; c < kN3; ++c)
-          if (c < C) tw[c >> 2] |= (uint32_t)trow[c] << (8 * (c & 3));
+        for (int c = 0; c < 8; ++c)
+          if (8 * hf + c < C) tw[c >> 2] |= (uint32_t)trow[c] << (8 * (c & 3));
       }
     }
     {
       const int j = tb->level[m];
       const int wm = tb->wm[m], hm = tb->hm[m];
-      GridSample gs;
-      if (LEARNED) learned_g0(M, P, j, x, y, wm, hm, valid, noise_on, nkey, W, row);
+      // half 0: G0, half 1: G1 (learned interpolation: three of G0's taps
+      // against the fourth and G1), the encoding and the constants
+      auto grid_rows = [&](int k) {
+        const int ck = k ? M.c1 : M.c0, s0 = k ? P.f0 : 0, ng = k ? P.f1 : P.f0;
+        if (!noise_on && (ck & 3) == 0 && ck <= kFastGridCh) {
+          const ntc_level& L = M.lv[j];
+          const float* base = use_copy ? (k ? A.noisy1[j] : A.noisy0[j])
+                                       : static_cast<const float*>(k ? L.grid1 : L.grid0);
+          const Taps t = bilinear_taps(x, y, wm, hm, k ? L.g1_w : L.g0_w, k ? L.g1_h : L.g0_h);
 #pragma unroll
-      for (int k = LEARNED ? 1 : 0; k < 2; ++k) {
-        const int ck = k ? M.c1 : M.c0;
-        if (!noise_on && (ck & 3) == 0 && ck <= kFastGridCh)
-          sample_grid_f32x4(M, j, k, x, y, wm, hm, gs, use_copy ? (k ? A.noisy1[j] : A.noisy0[j]) : nullptr);
-        else
+          for (int g = 0; g < kFastGridCh / 8; ++g)
+            if (g < ng) {
+              float v[8];
+              sample_group_f32(base, ck, t, g, v);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] = valid ? v[e] : 0.f;
+              if (F8) put_x8(W, P, row, s0 + g, v, 1.f / sa[0], false, am[0]);
+              else put_x(W, P, row, s0 + g, v);
+            }
+        } else {
+          GridSample gs;
           sample_grid<true>(M, j, k, x, y, wm, hm, noise_on && valid, nkey, gs);
-        const int g0 = k ? P.f0 : 0, ng = k ? P.f1 : P.f0;
 #pragma unroll
-        for (int g = 0; g < kGridPad / 8; ++g)
-          if (g < ng) {
-            float v[8];
+          for (int g = 0; g < kGridPad / 8; ++g)
+            if (g < ng) {
+              float v[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = valid ? gs.acc[8 * g + e] : 0.f;
-            if (F8) put_x8(W, P, row, g0 + g, v, 1.f / sa[0], false, am[0]);
-            else put_x(W, P, row, g0 + g, v);
-          }
+              for (int e = 0; e < 8; ++e) v[e] = valid ? gs.acc[8 * g + e] : 0.f;
+              if (F8) put_x8(W, P, row, s0 + g, v, 1.f / sa[0], false, am[0]);
+              else put_x(W, P, row, s0 + g, v);
+            }
+        }
+      };
+      if (LEARNED) {
+        if (hf == 0) learned_g0<0>(M, P, j, x, y, wm, hm, valid, noise_on, nkey, W, row);
+        else learned_g0<1>(M, P, j, x, y, wm, hm, valid, noise_on, nkey, W, row);
+        if (hf) grid_rows(1);
+      } else {
+        grid_rows(hf);
       }
+      if (hf) {
       struct Pe {
         float v[16];
         __device__ void operator()(int q, float t) { v[q] = t; }
@@ -1006,39 +1011,37 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
         for (int g = P.k_int / 8; g < P.k8 / 8; ++g)
           *reinterpret_cast<uint2*>(W + P.H1 + tc::canon_chunk(row, g >> 1, kRows) + (g & 1) * 8) =
               make_uint2(0u, 0u);
+      }
     }
-    if (A.target)
-      *reinterpret_cast<uint4*>(W + P.DZ3 + tc::canon_chunk(row, 1, kRows)) =
-          make_uint4(tw[0], tw[1], tw[2], tw[3]);
     tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kRows);
+    tc::bar_sync(bar_id, kPipe);
 
     // ---- layer 1 -----------------------------------------------------------------
-    if (row == 0) {
+    if (pw == 0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (F8) {
         issue_kmajor_f8(tD, sW + P.H1, lbo_a, sbase + P.w1_8, lbo64, P.k8 / 32, id64);
       } else {
         issue_kmajor(tD, sW + P.X, lbo_a, sbase + P.w1, lbo64, P.k_int / 16, id64, 0);
         for (int s = 0; s < P.k_int / 16; ++s)
-          tc::mma_f16(tD, tc::smem_desc(sW + xlo_group(P, 2 * s), lbo_a, 128),
-                      tc::smem_desc(sbase + P.w1 + 2 * s * lbo64, lbo64, 128), id64, 1);
+          tc::mma_f16(tD, tc::desc_of(tc::desc_lo(sW + xlo_group(P, 2 * s), lbo_a), 128),
+                      tc::desc_of(tc::desc_lo(sbase + P.w1 + 2 * s * lbo64, lbo64), 128), id64, 1);
       }
       tc::mma_commit(bar);
     }
-    if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+    wait_phase(bar, phase, bad);
     tc::fence_after_sync();
     if (F8)
       hidden_forward_f8<ACT>(tD + lane, sa[0] * sw[0], reinterpret_cast<const float*>(sm + P.bf),
-                             1.f / sa[1], W + P.H1, W + P.H2, W + P.G1, row, am[1]);
+                             1.f / sa[1], W + P.H1, W + P.H2, W + P.G1, row, hf, am[1]);
     else
-      hidden_forward<ACT>(tD + lane, W + P.H1, W + P.G1, W + P.H2, row);
+      hidden_forward<ACT>(tD + lane, W + P.H1, W + P.G1, W + P.H2, row, hf);
     tc::fence_before_sync();
     tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kRows);
+    tc::bar_sync(bar_id, kPipe);
 
     // ---- layer 2 -----------------------------------------------------------------
-    if (row == 0) {
+    if (pw == 0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (F8) {
         issue_kmajor_f8(tD, sW + P.H2, lbo_a, sbase + P.w2_8, lbo64, 2, id64);
@@ -1049,37 +1052,37 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
       }
       tc::mma_commit(bar);
     }
-    if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+    wait_phase(bar, phase, bad);
     tc::fence_after_sync();
     if (F8)
       hidden_forward_f8<ACT>(tD + lane, sa[1] * sw[1],
                              reinterpret_cast<const float*>(sm + P.bf) + kHidden, 1.f / sa[2],
-                             W + P.H2, W + P.S8, W + P.G2, row, am[2]);
+                             W + P.H2, W + P.S8, W + P.G2, row, hf, am[2]);
     else
-      hidden_forward<ACT>(tD + lane, W + P.H2, W + P.G2, P.h3 ? W + P.H3 : nullptr, row);
+      hidden_forward<ACT>(tD + lane, W + P.H2, W + P.G2, P.h3 ? W + P.H3 : nullptr, row, hf);
     tc::fence_before_sync();
     tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kRows);
+    tc::bar_sync(bar_id, kPipe);
 
     // ---- third hidden layer (Sec. 4.4) -------------------------------------------
     if (P.h3) {
-      if (row == 0) {
+      if (pw == 0 && tc::elect_one()) {
         tc::fence_after_sync();
         issue_kmajor(tD, sW + P.H2, lbo_a, sbase + P.wh, lbo64, 4, id64, 0);
         issue_kmajor(tD, sW + P.H3, lbo_a, sbase + P.wh, lbo64, 4, id64, 1);
         issue_kmajor(tD, sW + P.ONEa, lbo_a, sbase + P.wbh, lbo64, 1, id64, 1);
         tc::mma_commit(bar);
       }
-      if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+      wait_phase(bar, phase, bad);
       tc::fence_after_sync();
-      hidden_forward<ACT>(tD + lane, W + P.H3, W + P.G3, nullptr, row);
+      hidden_forward<ACT>(tD + lane, W + P.H3, W + P.G3, nullptr, row, hf);
       tc::fence_before_sync();
       tc::fence_proxy_async();
-      tc::bar_sync(bar_id, kRows);
+      tc::bar_sync(bar_id, kPipe);
     }
 
     // ---- layer 3, loss, dZ3 ----------------------------------------------------
-    if (row == 0) {
+    if (pw == 0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (F8) {
         issue_kmajor_f8(tD, sW + P.S8, lbo_a, sbase + P.w3_8, lbo16, 2, id16);
@@ -1089,108 +1092,97 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
       }
       tc::mma_commit(bar);
     }
-    if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+    wait_phase(bar, phase, bad);
     tc::fence_after_sync();
     {
-      float zv[16];
-      tc::tmem_ld16(tD + lane, zv);
+      // channels 8 hf .. 8 hf + 7
+      float zv[8];
+      tc::tmem_ld8(tD + lane + 8 * hf, zv);
       tc::tmem_ld_wait();
       if (F8) {
-        const float* b3 = reinterpret_cast<const float*>(sm + P.bf) + 2 * kHidden;
+        const float* b3 = reinterpret_cast<const float*>(sm + P.bf) + 2 * kHidden + 8 * hf;
 #pragma unroll
-        for (int c = 0; c < kN3; ++c) zv[c] = fmaf(zv[c], sa[2] * sw[2], b3[c]);
+        for (int c = 0; c < 8; ++c) zv[c] = fmaf(zv[c], sa[2] * sw[2], b3[c]);
       }
-      // the target texel (loss mode) or the upstream gradient row (dout mode)
-      float tgt[kN3];
-      if (A.target) {
-        const uint4 t4 = *reinterpret_cast<const uint4*>(W + P.DZ3 + tc::canon_chunk(row, 1, kRows));
-        const uint32_t tv[4] = {t4.x, t4.y, t4.z, t4.w};
+      float v[8];
 #pragma unroll
-        for (int c = 0; c < kN3; ++c) tgt[c] = (float)((tv[c >> 2] >> (8 * (c & 3))) & 0xFFu) * (1.f / 255.f);
-      } else {
-#pragma unroll
-        for (int c = 0; c < kN3; ++c) tgt[c] = (valid && c < C) ? A.dout[i * C + c] : 0.f;
-      }
-      float d[16];
-#pragma unroll
-      for (int c = 0; c < kN3; ++c) {
+      for (int c = 0; c < 8; ++c) {
         float g = 0.f;
-        if (valid && c < C) {
+        if (valid && 8 * hf + c < C) {
+          // the target texel (loss mode) or the upstream gradient row (dout mode)
+          const float tgt = A.target ? (float)((tw[c >> 2] >> (8 * (c & 3))) & 0xFFu) * (1.f / 255.f)
+                                     : A.dout[i * C + 8 * hf + c];
           // sigmoid; the fast division is within 2 ulp
           const float yc = M.out_act == NTC_OUT_IDENTITY ? zv[c] : __fdividef(1.f, 1.f + __expf(-zv[c]));
           if (A.target) {
-            const float e = yc - tgt[c];
+            const float e = yc - tgt;
             loss_acc = fmaf(e, e, loss_acc);
             g = M.out_act == NTC_OUT_IDENTITY ? 2.f * e : 2.f * e * yc * (1.f - yc);
           } else {
-            const float d = tgt[c] * dscale;
+            const float d = tgt * dscale;
             g = M.out_act == NTC_OUT_IDENTITY ? d : d * yc * (1.f - yc);
           }
         }
-        d[c] = g;
+        v[c] = g;
       }
-      float v0[8], v1[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) { v0[e] = d[e]; v1[e] = d[8 + e]; }
-      put_chunk(W + P.DZ3, row, 0, v0);
-      put_chunk(W + P.DZ3, row, 1, v1);
+      put_chunk(W + P.DZ3, row, hf, v);
     }
     tc::fence_before_sync();
     tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kRows);
+    tc::bar_sync(bar_id, kPipe);
 
     // ---- dHL = dZ3 W3; [dW3^T; db3] += [HL^T; 1] dZ3; then dZL over HL -------
-    if (row == 0) {
+    if (pw == 0 && tc::elect_one()) {
       tc::fence_after_sync();
       issue_kmn(tD, sW + P.DZ3, lbo_a, sbase + P.w3, (kN3 / 8) * 128, 1, id64 | idb);
       issue_mnmajor(tW3, sW + P.HL, sW + P.DZ3, id_w3, 1);
       tc::mma_commit(bar);
     }
-    if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+    wait_phase(bar, phase, bad);
     tc::fence_after_sync();
-    hidden_backward<ACT, F8>(tD + lane, W + (P.h3 ? P.G3 : P.G2), W + P.HL, row, sw[2]);
+    hidden_backward<ACT, F8>(tD + lane, W + (P.h3 ? P.G3 : P.G2), W + P.HL, row, hf, sw[2]);
     tc::fence_before_sync();
     tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kRows);
+    tc::bar_sync(bar_id, kPipe);
 
     // ---- third layer: dH2 = dZh Wh; [dWh dbh] += dZh^T [H2 | 1]; dZ2 over H2 --
     if (P.h3) {
-      if (row == 0) {
+      if (pw == 0 && tc::elect_one()) {
         tc::fence_after_sync();
         issue_kmn(tD, sW + P.H3, lbo_a, sbase + P.wh, lbo64, 4, id64 | idb);
         issue_mnmajor(tWh, sW + P.H3, sW + P.H2, id_w2, 1);
         tc::mma_commit(bar);
       }
-      if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+      wait_phase(bar, phase, bad);
       tc::fence_after_sync();
-      hidden_backward<ACT, F8>(tD + lane, W + P.G2, W + P.H2, row);
+      hidden_backward<ACT, F8>(tD + lane, W + P.G2, W + P.H2, row, hf);
       tc::fence_before_sync();
       tc::fence_proxy_async();
-      tc::bar_sync(bar_id, kRows);
+      tc::bar_sync(bar_id, kPipe);
     }
 
     // ---- dH1 = dZ2 W2; [dW2 db2] += dZ2^T [H1 | 1]; then dZ1 over H1 ----------
-    if (row == 0) {
+    if (pw == 0 && tc::elect_one()) {
       tc::fence_after_sync();
       issue_kmn(tD, sW + P.H2, lbo_a, sbase + P.w2, lbo64, 4, id64 | idb);
       issue_mnmajor(tW2, sW + P.H2, sW + P.H1, id_w2, 1);
       tc::mma_commit(bar);
     }
-    if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+    wait_phase(bar, phase, bad);
     tc::fence_after_sync();
-    hidden_backward<ACT, F8>(tD + lane, W + P.G1, W + P.H1, row, sw[1]);
+    hidden_backward<ACT, F8>(tD + lane, W + P.G1, W + P.H1, row, hf, sw[1]);
     tc::fence_before_sync();
     tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kRows);
+    tc::bar_sync(bar_id, kPipe);
 
     // ---- dX = dZ1 W1; [dW1 db1] += dZ1^T X ------------------------------------
-    if (row == 0) {
+    if (pw == 0 && tc::elect_one()) {
       tc::fence_after_sync();
       issue_kmn(tD, sW + P.H1, lbo_a, sbase + P.w1, lbo64, 4, id_dx);
       issue_mnmajor(tW1, sW + P.H1, sW + P.X, id_w1, 1);
       tc::mma_commit(bar);
     }
-    if (!wait_phase(bar, phase, bar_id)) { aborted = true; break; }
+    wait_phase(bar, phase, bad);
     tc::fence_after_sync();
     const bool staged = LEARNED || M.c0 > kFastGridCh || M.c1 > kFastGridCh;
     const bool vec_scatter = A.grids && !staged && (M.c0 & 3) == 0 && (M.c1 & 3) == 0;
@@ -1201,12 +1193,39 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
     const bool vec_staged = A.grids && staged && (M.c0 & 3) == 0 && M.c0 <= kFastGridCh &&
                             (M.c1 & 3) == 0 && M.c1 <= kFastGridCh &&
                             P.wg_bytes >= (uint32_t)(kRows * kDxStride * 4 + 4 * 32 * kScatMeta);
+    // this half's grid: the four taps' cell addresses and weights of the row's
+    // texel into its place of a warp's tap table
+    auto put_meta = [&](uint8_t* at) {
+      float* ga[4] = {nullptr, nullptr, nullptr, nullptr};
+      float wt[4] = {0.f, 0.f, 0.f, 0.f};
+      if (valid) {
+        const int j = tb->level[m];
+        const int wm = tb->wm[m], hm = tb->hm[m];
+        const ntc_level& L = M.lv[j];
+        const float gsc = F8 ? gscale * sw[0] : gscale;
+        if (float* g = hf ? A.g.grid1[j] : A.g.grid0[j]) {
+          const Taps t = bilinear_taps(x, y, wm, hm, hf ? L.g1_w : L.g0_w, hf ? L.g1_h : L.g0_h);
+#pragma unroll
+          for (int tp = 0; tp < 4; ++tp) {
+            ga[tp] = g + (size_t)t.cell[tp] * (hf ? M.c1 : M.c0);
+            wt[tp] = (LEARNED && hf == 0 ? 1.f : t.w[tp]) * gsc;
+          }
+        }
+      }
+      uint4* mq = reinterpret_cast<uint4*>(at);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const uint64_t a0 = reinterpret_cast<uint64_t>(ga[2 * e]), a1 = reinterpret_cast<uint64_t>(ga[2 * e + 1]);
+        mq[2 * hf + e] = make_uint4((uint32_t)a0, (uint32_t)(a0 >> 32), (uint32_t)a1, (uint32_t)(a1 >> 32));
+      }
+      mq[4 + hf] = make_uint4(__float_as_uint(wt[0]), __float_as_uint(wt[1]), __float_as_uint(wt[2]), __float_as_uint(wt[3]));
+    };
     if (A.grids && staged) {
       // dX row -> this thread's staging row (the operand tiles are free now),
       // then G0 per tap slot (weight 1; learned interpolation) or through
       // the bilinear taps, and G1 through the bilinear taps
       float* dxs = reinterpret_cast<float*>(W) + row * kDxStride;
-      for (int cb = 0; cb < P.dx_n; cb += 16) {
+      for (int cb = 16 * hf; cb < P.dx_n; cb += 32) {
         float v[16];
         tc::tmem_ld16(tD + lane + cb, v);
         tc::tmem_ld_wait();
@@ -1222,68 +1241,37 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
         // 4 (j % 4) .. +3 texel by texel, once per run of equal cells
         const int ln = tid & 31, wq = warp & 3;
         uint8_t* mbase = W + kRows * kDxStride * 4 + wq * 32 * kScatMeta;
-        {
-          float* ga[8];
-          float wt[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) { ga[e] = nullptr; wt[e] = 0.f; }
-          if (valid) {
-            const int j = tb->level[m];
-            const int wm = tb->wm[m], hm = tb->hm[m];
-            const ntc_level& L = M.lv[j];
-            const float gsc = F8 ? gscale * sw[0] : gscale;
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              float* g = k ? A.g.grid1[j] : A.g.grid0[j];
-              if (!g) continue;
-              const int c = k ? M.c1 : M.c0;
-              const Taps t = bilinear_taps(x, y, wm, hm, k ? L.g1_w : L.g0_w, k ? L.g1_h : L.g0_h);
-#pragma unroll
-              for (int tp = 0; tp < 4; ++tp) {
-                ga[4 * k + tp] = g + (size_t)t.cell[tp] * c;
-                wt[4 * k + tp] = (LEARNED && k == 0 ? 1.f : t.w[tp]) * gsc;
-              }
-            }
-          }
-          uint4* mq = reinterpret_cast<uint4*>(mbase + ln * kScatMeta);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const uint64_t a0 = reinterpret_cast<uint64_t>(ga[2 * e]), a1 = reinterpret_cast<uint64_t>(ga[2 * e + 1]);
-            mq[e] = make_uint4((uint32_t)a0, (uint32_t)(a0 >> 32), (uint32_t)a1, (uint32_t)(a1 >> 32));
-          }
-          mq[4] = make_uint4(__float_as_uint(wt[0]), __float_as_uint(wt[1]), __float_as_uint(wt[2]), __float_as_uint(wt[3]));
-          mq[5] = make_uint4(__float_as_uint(wt[4]), __float_as_uint(wt[5]), __float_as_uint(wt[6]), __float_as_uint(wt[7]));
-        }
-        __syncwarp();
+        put_meta(mbase + ln * kScatMeta);
+        tc::bar_sync(bar_id, kPipe);
         const int k = ln >> 4, slot = ln >> 2, q = ln & 3;
         if (4 * q < (k ? M.c1 : M.c0)) {
           const int col = (k ? 8 * P.f0 : (LEARNED ? ((ln >> 2) & 3) * M.c0 : 0)) + 4 * q;
-          const float* dx0 = reinterpret_cast<const float*>(W) + (32 * wq) * kDxStride + col;
-          if (merge) scatter_lane<true>(mbase, dx0, kDxStride, slot, q);
-          else scatter_lane<false>(mbase, dx0, kDxStride, slot, q);
+          const float* dx0 = reinterpret_cast<const float*>(W) + (32 * wq + 16 * hf) * kDxStride + col;
+          const uint8_t* m0 = mbase + 16 * hf * kScatMeta;
+          if (merge) scatter_lane<true>(m0, dx0, kDxStride, slot, q);
+          else scatter_lane<false>(m0, dx0, kDxStride, slot, q);
         }
-      } else if (valid) {
+      } else {
+        tc::bar_sync(bar_id, kPipe);  // both halves of the row are staged
+        const float* dxs = reinterpret_cast<const float*>(W) + row * kDxStride;
         const int j = tb->level[m];
         const int wm = tb->wm[m], hm = tb->hm[m];
         const ntc_level& L = M.lv[j];
-        if (float* g = A.g.grid0[j])
+        float* g = valid ? (hf ? A.g.grid1[j] : A.g.grid0[j]) : nullptr;
+        if (g && hf == 0)
           scatter_taps(g, M.c0, bilinear_taps(x, y, wm, hm, L.g0_w, L.g0_h), dxs,
                        LEARNED ? M.c0 : 0, !LEARNED, F8 ? gscale * sw[0] : gscale);
-        if (float* g = A.g.grid1[j])
+        if (g && hf == 1)
           scatter_taps(g, M.c1, bilinear_taps(x, y, wm, hm, L.g1_w, L.g1_h), dxs + 8 * P.f0, 0,
                        true, F8 ? gscale * sw[0] : gscale);
       }
       // the staging rows ran over the constant-one tiles: once every row has
       // been read, each thread writes its row's chunks back
-      tc::bar_sync(bar_id, kRows);
-      const uint4 one = make_uint4(tc::pack_f16x2(1.f, 1.f), 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(W + P.ONEa + tc::canon_chunk(row, 0, kRows)) = one;
-      *reinterpret_cast<uint4*>(W + P.ONEa + tc::canon_chunk(row, 1, kRows)) = make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(W + P.ONEb + tc::canon_chunk(row, 0, kRows)) = one;
-      if (P.h3) {
-        *reinterpret_cast<uint4*>(W + P.ONEc + tc::canon_chunk(row, 0, kRows)) = one;
-        *reinterpret_cast<uint4*>(W + P.ONEc + tc::canon_chunk(row, 1, kRows)) = make_uint4(0, 0, 0, 0);
-      }
+      tc::bar_sync(bar_id, kPipe);
+      const uint4 one = make_uint4(tc::pack_f16x2(1.f, 1.f), 0u, 0u, 0u), zero = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4*>(W + P.ONEa + tc::canon_chunk(row, hf, kRows)) = hf ? zero : one;
+      if (!hf) *reinterpret_cast<uint4*>(W + P.ONEb + tc::canon_chunk(row, 0, kRows)) = one;
+      if (P.h3) *reinterpret_cast<uint4*>(W + P.ONEc + tc::canon_chunk(row, hf, kRows)) = hf ? zero : one;
     } else if (vec_scatter) {
       // Coalesced scatter (grids of 4k <= 16 channels): each warp stages
       // its 32 texels' dX rows, cell addresses and tap weights in its 8 KB
@@ -1296,91 +1284,46 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
       uint8_t* ws = W + (warp & 3) * kScatWarp;
       float* dxr = reinterpret_cast<float*>(ws) + ln * kScatDx;
       uint8_t* mr = ws + 32 * kScatDx * 4 + ln * kScatMeta;
-#pragma unroll
-      for (int cb = 0; cb < 32; cb += 16) {
+      {
         float v[16];
-        tc::tmem_ld16(tD + lane + cb, v);
+        tc::tmem_ld16(tD + lane + 16 * hf, v);
         tc::tmem_ld_wait();
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          *reinterpret_cast<float4*>(dxr + cb + 4 * q) =
+          *reinterpret_cast<float4*>(dxr + 16 * hf + 4 * q) =
               make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
-      {
-        float* ga[8];
-        float wt[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) { ga[e] = nullptr; wt[e] = 0.f; }
-        if (valid) {
-          const int j = tb->level[m];
-          const int wm = tb->wm[m], hm = tb->hm[m];
-          const ntc_level& L = M.lv[j];
-          const float gsc = F8 ? gscale * sw[0] : gscale;
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            float* g = k ? A.g.grid1[j] : A.g.grid0[j];
-            if (!g) continue;
-            const int c = k ? M.c1 : M.c0;
-            const Taps t = bilinear_taps(x, y, wm, hm, k ? L.g1_w : L.g0_w, k ? L.g1_h : L.g0_h);
-#pragma unroll
-            for (int tp = 0; tp < 4; ++tp) {
-              ga[4 * k + tp] = g + (size_t)t.cell[tp] * c;
-              wt[4 * k + tp] = t.w[tp] * gsc;
-            }
-          }
-        }
-        uint4* mq = reinterpret_cast<uint4*>(mr);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const uint64_t a0 = reinterpret_cast<uint64_t>(ga[2 * e]), a1 = reinterpret_cast<uint64_t>(ga[2 * e + 1]);
-          mq[e] = make_uint4((uint32_t)a0, (uint32_t)(a0 >> 32), (uint32_t)a1, (uint32_t)(a1 >> 32));
-        }
-        mq[4] = make_uint4(__float_as_uint(wt[0]), __float_as_uint(wt[1]), __float_as_uint(wt[2]), __float_as_uint(wt[3]));
-        mq[5] = make_uint4(__float_as_uint(wt[4]), __float_as_uint(wt[5]), __float_as_uint(wt[6]), __float_as_uint(wt[7]));
-      }
-      __syncwarp();
+      put_meta(mr);
+      tc::bar_sync(bar_id, kPipe);
       {
         const int k = ln >> 4, slot = ln >> 2, q = ln & 3;
         const int col = (k ? 8 * P.f0 : 0) + 4 * q;
         if (4 * q < (k ? M.c1 : M.c0)) {
-          const float* dx0 = reinterpret_cast<const float*>(ws) + col;
-          const uint8_t* m0 = ws + 32 * kScatDx * 4;
+          const float* dx0 = reinterpret_cast<const float*>(ws) + 16 * hf * kScatDx + col;
+          const uint8_t* m0 = ws + 32 * kScatDx * 4 + 16 * hf * kScatMeta;
           if (merge) scatter_lane<true>(m0, dx0, kScatDx, slot, q);
           else scatter_lane<false>(m0, dx0, kScatDx, slot, q);
         }
       }
       // the staging ran over ONEa: once every warp of the pipeline is done
       // with its rows, each thread writes its row's chunks back
-      tc::bar_sync(bar_id, kRows);
-      const uint4 one = make_uint4(tc::pack_f16x2(1.f, 1.f), 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(W + P.ONEa + tc::canon_chunk(row, 0, kRows)) = one;
-      *reinterpret_cast<uint4*>(W + P.ONEa + tc::canon_chunk(row, 1, kRows)) = make_uint4(0, 0, 0, 0);
+      tc::bar_sync(bar_id, kPipe);
+      const uint4 one = make_uint4(tc::pack_f16x2(1.f, 1.f), 0u, 0u, 0u), zero = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4*>(W + P.ONEa + tc::canon_chunk(row, hf, kRows)) = hf ? zero : one;
     } else if (A.grids) {
-      // dX slots: G0 at columns 0.., G1 at 8 * f0.. (f0 is 1 or 2)
-      float d[32], dg0[16], dg1[16];
-      {
-        float lo[16], hi[16];
-        tc::tmem_ld16(tD + lane, lo);
-        tc::tmem_ld16(tD + lane + 16, hi);
-        tc::tmem_ld_wait();
-#pragma unroll
-        for (int e = 0; e < 16; ++e) { d[e] = lo[e]; d[16 + e] = hi[e]; }
-      }
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        dg0[e] = d[e];
-        dg1[e] = P.f0 == 1 ? d[8 + e] : d[16 + e];
-      }
+      // dX slots: G0 at columns 0.., G1 at 8 * f0.. (f0 is 1 or 2); a half
+      // scatters one grid
+      float d[16];
+      tc::tmem_ld16(tD + lane + (hf ? 8 * P.f0 : 0), d);
+      tc::tmem_ld_wait();
       if (valid) {
         const int j = tb->level[m];
         const int wm = tb->wm[m], hm = tb->hm[m];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const ntc_level& L = M.lv[j];
-          float* g = k ? A.g.grid1[j] : A.g.grid0[j];
-          if (!g) continue;
-          const int c = k ? M.c1 : M.c0;
-          const Taps t = bilinear_taps(x, y, wm, hm, k ? L.g1_w : L.g0_w, k ? L.g1_h : L.g0_h);
+        const ntc_level& L = M.lv[j];
+        float* g = hf ? A.g.grid1[j] : A.g.grid0[j];
+        const int c = hf ? M.c1 : M.c0;
+        if (g) {
+          const Taps t = bilinear_taps(x, y, wm, hm, hf ? L.g1_w : L.g0_w, hf ? L.g1_h : L.g0_h);
 #pragma unroll
           for (int tp = 0; tp < 4; ++tp) {
             const float wgt = t.w[tp] * (F8 ? gscale * sw[0] : gscale);
@@ -1388,16 +1331,14 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
             if ((c & 3) == 0) {
 #pragma unroll
               for (int c4 = 0; c4 < 4; ++c4)
-                if (4 * c4 < c) {
-                  const float* d = k ? dg1 : dg0;
+                if (4 * c4 < c)
                   atomicAdd(reinterpret_cast<float4*>(gp) + c4,
                             make_float4(d[4 * c4] * wgt, d[4 * c4 + 1] * wgt, d[4 * c4 + 2] * wgt,
                                         d[4 * c4 + 3] * wgt));
-                }
             } else {
 #pragma unroll
               for (int ch = 0; ch < kFastGridCh; ++ch)
-                if (ch < c) atomicAdd(gp + ch, (k ? dg1[ch] : dg0[ch]) * wgt);
+                if (ch < c) atomicAdd(gp + ch, d[ch] * wgt);
             }
           }
         }
@@ -1405,15 +1346,16 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
     }
     tc::fence_before_sync();
     if (staged || vec_scatter) tc::fence_proxy_async();  // restored constants, read by the next tile's MMAs
-    tc::bar_sync(bar_id, kRows);  // the next tile's features overwrite the operand tiles
+    // the next tile's features overwrite the operand tiles
+    if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
   }
 
   // ---- every MMA of this pipeline has completed (bounded) ---------------------
-  if (row == 0) {
+  if (pw == 0 && tc::elect_one()) {
     tc::fence_after_sync();
     tc::mma_commit(&fin[wg]);
-    if (!tc::mbar_wait(&fin[wg], fin_phase, kWaitLimit)) aborted = true;
-    if (aborted) abort_any = 1;
+    if (!tc::mbar_wait(&fin[wg], fin_phase, kWaitLimit)) bad = true;
+    if (bad) abort_any = 1;
   }
   fin_phase ^= 1;
   tc::fence_before_sync();
@@ -1425,15 +1367,17 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
   const int wq = warp & 3;  // lane quarter of this warp: rows 32 wq .. 32 wq + 31
   const int r = 32 * wq + (tid & 31);
   if (!abort_any && (BATCHED || (int64_t)blockIdx.x * NWG < t_hi)) {
-    // flush jobs 0 dW1, 1 dW2, 2 dW3, 3 dWh, one warpgroup each (round robin)
-    for (int job = wg; job < (P.h3 ? 4 : 3); job += NWG) {
+    // flush jobs 0 dW1, 1 dW2, 2 dW3, 3 dWh, the wide ones in two column
+    // halves; four warps each (round robin)
+    for (int j2 = tid / kRows; j2 < (P.h3 ? 8 : 6); j2 += 2 * NWG) {
+      const int job = j2 >> 1, part = j2 & 1;
       if (job == 0 && wq < 2) {
         // [dW1 db1]: row r, X columns (the head constant-one slot gives db1
         // r); four slots that map to four consecutive, 16-byte aligned user
         // columns leave as one vector reduction
         float* gw = A.g.w[0];
 #pragma unroll 1
-        for (int cb = 0; cb < P.k_int; cb += 16) {
+        for (int cb = 16 * part; cb < P.k_int; cb += 32) {
           float v[16];
           tc::tmem_ld16(tW1 + lane + cb, v);
           tc::tmem_ld_wait();
@@ -1467,7 +1411,7 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
         const float gsw = gs * (job == 1 ? sa[1] : 1.f);  // FP8: H1 was held in units of s_a1
         const bool vec = gw && (reinterpret_cast<uintptr_t>(gw + r * kHidden) & 15) == 0;
 #pragma unroll 1
-        for (int cb = 0; cb < kHidden + 16; cb += 16) {
+        for (int cb = 16 * part; cb < kHidden + 16; cb += 32) {
           float v[16];
           tc::tmem_ld16(ta + lane + cb, v);
           tc::tmem_ld_wait();
@@ -1486,7 +1430,7 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
             }
           }
         }
-      } else if (job == 2 && wq < 3) {
+      } else if (job == 2 && part == 0 && wq < 3) {
         // [dW3^T; db3]: row r < 64 -> dW3[:, r]; row 64 -> db3
         float v[16];
         tc::tmem_ld16(tW3 + lane, v);
@@ -1520,7 +1464,7 @@ __global__ void __launch_bounds__(kRows* NWG, 1) train_tc_kernel(const ntc_mater
   __syncthreads();
   if (tid == 0) {
     float s = 0.f;
-    for (int w = 0; w < NWG * 4; ++w) s += red[w];
+    for (int w = 0; w < NWG * 8; ++w) s += red[w];
     if (A.loss) atomicAdd(A.loss, s * A.loss_scale);
     if (abort_any) atomicExch(status, NTC_ERR_TIMEOUT);
   }
@@ -1551,7 +1495,7 @@ cudaError_t launch_t(const ntc_material& m, const BwdArgs& a, const TrainBatchDe
   const int64_t cap = sm_count();
   const int grid = (int)(ctas < cap ? ctas : cap);
   train_tc_kernel<ACT, LEARNED, NWG, BATCHED, F8>
-      <<<grid, kRows * NWG, smem, s>>>(m, a, hb, k_lay, dx_lay, status_word());
+      <<<grid, kPipe * NWG, smem, s>>>(m, a, hb, k_lay, dx_lay, status_word());
   return cudaGetLastError();
 }
 
@@ -1566,11 +1510,18 @@ int pipelines_for(const ntc_material& m, int k_lay, int dx_lay) {
 }
 int train_pipelines(const ntc_material& m) { return pipelines_for(m, 0, 0); }
 
+// Pipelines per CTA: the autotuner's choice (a.pipelines), else by the call.
+// Independent texels: two (their random gathers and reductions want the L1
+// that a third pipeline's tiles take, and 128 registers a thread: 2^18 texels
+// of a 2048^2 x 12 material 104 us against 112 with three); crops, whose
+// neighbours share cells: three where they fit (83 -> 79 us); a call with no
+// more tiles than SMs: one.
 template <int ACT, bool LEARNED, bool BATCHED, bool F8>
 cudaError_t launch_n(const ntc_material& m, const BwdArgs& a, const TrainBatchDev* hb,
                      int64_t tiles, int k_lay, int dx_lay, cudaStream_t s) {
-  int np = pipelines_for(m, k_lay, dx_lay);
-  if (a.pipelines > 0 && a.pipelines < np) np = a.pipelines;  // the autotuner's choice
+  const int most = pipelines_for(m, k_lay, dx_lay);
+  const int want = a.pipelines > 0 ? a.pipelines : (tiles <= sm_count() ? 1 : (a.crops ? 3 : 2));
+  const int np = want < most ? want : most;
   switch (np) {
     case 3: return launch_t<ACT, LEARNED, 3, BATCHED, F8>(m, a, hb, tiles, k_lay, dx_lay, s);
     case 2: return launch_t<ACT, LEARNED, 2, BATCHED, F8>(m, a, hb, tiles, k_lay, dx_lay, s);
