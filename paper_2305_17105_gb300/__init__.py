@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 
 import numpy as np
 import torch
@@ -281,30 +282,24 @@ class Material:
 
     @property
     def struct(self) -> ntc_material:
-        s = ntc_material()
-        s.width, s.height, s.channels, s.mips, s.levels = (self.width, self.height, self.channels,
-                                                           self.mips, self.levels)
-        s.c0, s.c1, s.bits0, s.bits1 = self.c0, self.c1, self.bits0, self.bits1
-        s.q0, s.q1 = self.q0, self.q1
-        s.encoding, s.k_in, s.hidden = self.encoding, self.k_in, HIDDEN
-        s.act, s.out_act, s.precision = self.act, self.out_act, self.precision
-        s.interp0 = self.interp0
-        for j in range(self.levels):
-            g0, g1 = self.grids0[j], self.grids1[j]
-            s.lv[j].g0_h, s.lv[j].g0_w = g0.shape[0], g0.shape[1]
-            s.lv[j].g1_h, s.lv[j].g1_w = g1.shape[0], g1.shape[1]
-            s.lv[j].grid0, s.lv[j].grid1 = g0.data_ptr(), g1.data_ptr()
-        w, b, wh, bh = _layers(self.weights), _layers(self.biases), None, None
-        for l in range(3):
-            s.w[l] = w[0][l].data_ptr()
-            s.b[l] = b[0][l].data_ptr()
-        s.hidden_layers = len(self.weights) - 1
+        # packed in one go: setting some 60 ctypes fields one by one was half
+        # of the host time of a small call
+        w, b, wh, bh = _layers(self.weights), _layers(self.biases), 0, 0
         if w[1] is not None:
-            s.w_h3, s.b_h3 = w[1].data_ptr(), b[1].data_ptr()
-        s.scale = self.scale.data_ptr() if self.scale is not None else None
-        if self.codebook0 is not None:
-            s.vq_books, s.codebook0 = self.codebook0.shape[0], self.codebook0.data_ptr()
-        return s
+            wh, bh = w[1].data_ptr(), b[1].data_ptr()
+        lv = []
+        for g0, g1 in zip(self.grids0, self.grids1):
+            s0, s1 = g0.shape, g1.shape
+            lv += (s0[1], s0[0], s1[1], s1[0], g0.data_ptr(), g1.data_ptr())
+        lv += (0,) * (6 * (MAX_LEVELS - self.levels))
+        cb = self.codebook0
+        return ntc_material.from_buffer_copy(_MATERIAL_FMT.pack(
+            self.width, self.height, self.channels, self.mips, self.levels, self.c0, self.c1,
+            self.bits0, self.bits1, self.q0, self.q1, self.encoding, self.k_in, HIDDEN, self.act,
+            self.out_act, self.precision, self.interp0, *lv, *[x.data_ptr() for x in w[0]],
+            *[x.data_ptr() for x in b[0]], self.scale.data_ptr() if self.scale is not None else 0,
+            len(self.weights) - 1, wh, bh, 0 if cb is None else cb.shape[0],
+            0 if cb is None else cb.data_ptr()))
 
     def with_(self, **kw) -> "Material":
         m = Material.__new__(Material)
@@ -313,6 +308,12 @@ class Material:
         if "grids0" in kw:
             m.encoding = GRID_PACKED if m.grids0[0].dtype == torch.uint8 else GRID_F32
         return m
+
+
+# ntc_material's fields in order, with native alignment (the padding bytes in
+# front of the pointers included)
+_MATERIAL_FMT = struct.Struct("@9i2f7i" + "4i2P" * MAX_LEVELS + "3P3PPi2PiP")
+assert _MATERIAL_FMT.size == C.sizeof(ntc_material)
 
 
 def _out_dtype(t: torch.Tensor) -> int:
@@ -841,7 +842,8 @@ class NTCDecodeFunction(torch.autograd.Function):
     def backward(ctx, dy):
         uvl, *tensors = ctx.saved_tensors
         L, nl = ctx.L, ctx.nl
-        grads = [torch.zeros_like(t) for t in tensors]
+        grads = [torch.empty_like(t) for t in tensors]
+        torch._foreach_zero_(grads)  # one launch for all of them
         gs = grads_struct(ctx.mat, grads[:L], grads[L:2 * L], grads[2 * L:2 * L + nl],
                           grads[2 * L + nl:2 * L + 2 * nl])
         ntc_backward(ctx.mat, uvl, dy.contiguous().float(), gs, flags=ctx.flags,

@@ -4,16 +4,22 @@
 // the sampler and the MLP input rows.
 #include <math.h>
 
+#include <atomic>
+
 #include "ntc_device.cuh"
 #include "ntc_internal.h"
 #include "tc_ptx.cuh"
 
 namespace ntc {
 
+// The current device's SM count, asked for once per device.
 int sm_count() {
+  static std::atomic<int> known[64];
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
   if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
+  if (n > 0 && dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
   return n > 0 ? n : 1;
 }
 

@@ -155,7 +155,14 @@ std::string tune_key(const char* kind, const ntc_material& m, int filter, int ou
   return std::string(buf);
 }
 
-int tune_lookup(const std::string& key) {
+// The recorded choice for a call (0: none); the key is only formed when the
+// cache holds anything.
+int tune_lookup(const char* kind, const ntc_material& m, int filter, int out_dtype, int64_t n) {
+  {
+    std::lock_guard<std::mutex> lock(g_tune_mu);
+    if (g_tune.empty()) return 0;
+  }
+  const std::string key = tune_key(kind, m, filter, out_dtype, n);
   std::lock_guard<std::mutex> lock(g_tune_mu);
   auto it = g_tune.find(key);
   return it == g_tune.end() ? 0 : it->second;
@@ -195,7 +202,7 @@ int decode_impl(const ntc_material* m, const float* uvl, int64_t n, void* out, i
                                                noise_step, s),
                        "decode (FP32 CUDA cores)");
   int nwg = g_decode_nwg.load();  // ntc_set_decode_warpgroups, else the autotuner's choice
-  if (nwg == 0) nwg = tune_lookup(tune_key("decode", *m, filter, out_dtype, n));
+  if (nwg == 0) nwg = tune_lookup("decode", *m, filter, out_dtype, n);
   return cuda_status(ntc::launch_decode_tc(*m, uvl, n, out, out_dtype, filter,
                                            ntc::jitter_key(noise_seed, noise_step), s, nwg),
                      "decode (tcgen05)");
@@ -656,7 +663,7 @@ static int plan_train_step(const ntc_material* m, const ntc_trainer* tr, const n
   b.crops = (flags & NTC_FLAG_CROPS) != 0;
   sp.vq = vq;
   sp.simt = use_simt(m, flags);
-  b.pipelines = sp.simt ? 0 : tune_lookup(tune_key("train", *m, b.crops ? 1 : 0, 0, batch));
+  b.pipelines = sp.simt ? 0 : tune_lookup("train", *m, b.crops ? 1 : 0, 0, batch);
   sp.cb_seg = cb_seg;
   // With the noisy scratch: one dense noise pass, and the fused step reads
   // the noisy grids at the same offsets of the scratch.
