@@ -54,19 +54,6 @@ int read_status_word(int reset) {
 
 namespace {
 
-// The noise of channels ch and ch + 1 (ch even) of a cell: both come from
-// the same 64-bit draw (the values noise_of gives for each).
-__device__ __forceinline__ float2 noise_pair_of(uint64_t key, int level, int grid, int cell,
-                                                int ch, int c, float q) {
-  const uint64_t pairs = (uint64_t)((c + 1) >> 1);
-  const uint64_t counter = ((uint64_t)(2 * level + grid) << 40) |
-                           ((uint64_t)cell * pairs + (uint64_t)(ch >> 1));
-  const uint64_t h = splitmix64(key ^ counter);
-  const uint32_t e = (uint32_t)(h >> 40), o = (uint32_t)((h >> 16) & 0xFFFFFFu);
-  return make_float2(((float)e * (1.0f / 16777216.0f) - 0.5f) * q,
-                     ((float)o * (1.0f / 16777216.0f) - 0.5f) * q);
-}
-
 // One Adam step (Kingma & Ba, bias-corrected) at the device step counter t,
 // learning rate lr0 (1 + cos(pi t / T)) / 2 per group, then the grid clamp
 // to [-(N-1)/2 Q, N/2 Q] (Sec. 4.2: clamp after the update).  The gradient is
@@ -139,9 +126,9 @@ __device__ __forceinline__ void adam_seg_block(const AdamArgs& A, const AdamSeg&
         // even channel counts: elements (first, first+1) and (first+2,
         // first+3) are channel pairs of one cell, one draw each
         const int64_t cell0 = first / c, cell1 = (first + 2) / c;
-        const float2 n0 = noise_pair_of(nkey, S.noise_level, S.noise_grid, (int)cell0,
+        const float2 n0 = noise_pair(nkey, S.noise_level, S.noise_grid, (int)cell0,
                                         (int)(first - cell0 * c), c, S.noise_q);
-        const float2 n1 = noise_pair_of(nkey, S.noise_level, S.noise_grid, (int)cell1,
+        const float2 n1 = noise_pair(nkey, S.noise_level, S.noise_grid, (int)cell1,
                                         (int)(first + 2 - cell1 * c), c, S.noise_q);
         nv = make_float4(po.x + n0.x, po.y + n0.y, po.z + n1.x, po.w + n1.y);
       } else {

@@ -99,6 +99,11 @@ __device__ __forceinline__ int stochastic_coord(float u, int w, uint32_t b24) {
   return wrap_texel((int)floorf(p), w);
 }
 
+// 1 / w of a power of two w >= 1 (a mip side), exactly.
+__device__ __forceinline__ float pow2_inverse(int w) {
+  return __int_as_float((127 - (31 - __clz(w))) << 23);
+}
+
 // Bilinear taps of a gw x gh grid for texel (x, y) of a wm x hm mip
 // (Sec. 4.3.1): texel centre (x + 1/2)/wm maps to p = centre * gw - 1/2 in
 // cell-centre coordinates; taps clamp to the grid edge.  With power-of-two
@@ -108,8 +113,8 @@ struct Taps {
   float w[4];
 };
 __device__ __forceinline__ Taps bilinear_taps(int x, int y, int wm, int hm, int gw, int gh) {
-  const float px = ((float)x + 0.5f) / (float)wm * (float)gw - 0.5f;
-  const float py = ((float)y + 0.5f) / (float)hm * (float)gh - 0.5f;
+  const float px = ((float)x + 0.5f) * pow2_inverse(wm) * (float)gw - 0.5f;
+  const float py = ((float)y + 0.5f) * pow2_inverse(hm) * (float)gh - 0.5f;
   const float fx0 = floorf(px), fy0 = floorf(py);
   const float fx = px - fx0, fy = py - fy0;
   int ix0 = (int)fx0, iy0 = (int)fy0;
@@ -161,6 +166,19 @@ __device__ __forceinline__ float noise_of(uint64_t key, int level, int grid, int
   return ((float)b24 * (1.0f / 16777216.0f) - 0.5f) * q;
 }
 
+// The noise of channels ch and ch + 1 (ch even) of a cell: both come from
+// the same draw (the values noise_of gives for each).
+__device__ __forceinline__ float2 noise_pair(uint64_t key, int level, int grid, int cell, int ch,
+                                             int c, float q) {
+  const uint64_t pairs = (uint64_t)((c + 1) >> 1);
+  const uint64_t counter = ((uint64_t)(2 * level + grid) << 40) |
+                           ((uint64_t)cell * pairs + (uint64_t)(ch >> 1));
+  const uint64_t h = splitmix64(key ^ counter);
+  const uint32_t e = (uint32_t)(h >> 40), o = (uint32_t)((h >> 16) & 0xFFFFFFu);
+  return make_float2(((float)e * (1.0f / 16777216.0f) - 0.5f) * q,
+                     ((float)o * (1.0f / 16777216.0f) - 0.5f) * q);
+}
+
 // Packed cell of up to 16 bytes.
 struct Cell {
   uint64_t lo, hi;
@@ -204,57 +222,43 @@ __host__ __device__ __forceinline__ int cell_bytes(int c, int bits) {
 }
 
 // ---------------------------------------------------------------------------
-// Features of one grid at texel (x, y) of mip m: acc[ch] = sum_t w_t g_t[ch].
+// Bilinear features of one grid: sum_t w_t g_t[ch] over the four taps, in
+// order, as fused multiply-adds.  The channels are walked four at a time in a
+// rolled loop, out(ch, v) receiving channels ch .. ch + 3 (those at or beyond
+// the grid's count are zero): unrolled over every channel, width and form, the
+// FP32 kernels' code reached 320 KB, and a call spent most of its time
+// fetching it (65,536 queries of a 256^2 x 8 material, cold: 43 us, of which
+// the FMA pipe worked 8).
 // ---------------------------------------------------------------------------
-struct GridSample {
-  float acc[kGridPad];  // channels >= c are zero
-};
-
-// Vector-quantised G0 (vq_books > 0): the c0 features of cell `cell` of
-// level j, the sum of the codebook entries its indices select.
-__device__ __forceinline__ void vq_cell(const ntc_material& M, int j, int cell,
-                                        float (&v)[kMaxGridCh]) {
-  const uint8_t* ib = static_cast<const uint8_t*>(M.lv[j].grid0) + (size_t)cell * M.vq_books;
-#pragma unroll
-  for (int ch = 0; ch < kMaxGridCh; ++ch) v[ch] = 0.f;
-  for (int b = 0; b < M.vq_books; ++b) {
-    const float* e = M.codebook0 + ((size_t)b * 256 + ib[b]) * M.c0;
-    if ((M.c0 & 3) == 0) {  // rows of 4k values: float4 reads
-#pragma unroll
-      for (int q4 = 0; q4 < kMaxGridCh / 4; ++q4)
-        if (4 * q4 < M.c0) {
-          const float4 f = __ldg(reinterpret_cast<const float4*>(e) + q4);
-          v[4 * q4] += f.x; v[4 * q4 + 1] += f.y; v[4 * q4 + 2] += f.z; v[4 * q4 + 3] += f.w;
-        }
-    } else {
-#pragma unroll
-      for (int ch = 0; ch < kMaxGridCh; ++ch)
-        if (ch < M.c0) v[ch] += __ldg(e + ch);
-    }
-  }
-}
-
 // F32: the grids are NTC_GRID_F32 and not vector-quantised (the trainers).
-template <bool F32 = false>
-__device__ __forceinline__ void sample_grid(const ntc_material& M, int j, int k, int x, int y,
-                                            int wm, int hm, bool noise, uint64_t nkey,
-                                            GridSample& gs, Taps* taps_out = nullptr) {
+template <bool F32, class Out>
+__device__ __forceinline__ void grid_quads(const ntc_material& M, int j, int k, const Taps& t, bool noise,
+                                           uint64_t nkey, Out out) {
   const ntc_level& L = M.lv[j];
-  const int gw = k ? L.g1_w : L.g0_w, gh = k ? L.g1_h : L.g0_h;
   const int c = k ? M.c1 : M.c0;
   const float q = k ? M.q1 : M.q0;
-  const Taps t = bilinear_taps(x, y, wm, hm, gw, gh);
-  if (taps_out) *taps_out = t;
-#pragma unroll
-  for (int ch = 0; ch < kGridPad; ++ch) gs.acc[ch] = 0.f;
+  const void* base = k ? L.grid1 : L.grid0;
   if (!F32 && k == 0 && M.vq_books > 0) {
+    // vector-quantised G0: the c0 features of a cell are the sum of the
+    // codebook entries that its indices select
+    const uint8_t* ib = static_cast<const uint8_t*>(base);
+#pragma unroll 1
+    for (int ch = 0; ch < c; ch += 4) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int tp = 0; tp < 4; ++tp) {
-      float v[kMaxGridCh];
-      vq_cell(M, j, t.cell[tp], v);
+      for (int tp = 0; tp < 4; ++tp) {
+        float e[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int b = 0; b < M.vq_books; ++b) {
+          const float* r = M.codebook0 + ((size_t)b * 256 + ib[(size_t)t.cell[tp] * M.vq_books + b]) * c + ch;
 #pragma unroll
-      for (int ch = 0; ch < kMaxGridCh; ++ch)
-        if (ch < c) gs.acc[ch] = fmaf(t.w[tp], v[ch], gs.acc[ch]);
+          for (int i = 0; i < 4; ++i)
+            if (ch + i < c) e[i] += __ldg(r + i);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = fmaf(t.w[tp], e[i], v[i]);
+      }
+      out(ch, v);
     }
     return;
   }
@@ -262,48 +266,71 @@ __device__ __forceinline__ void sample_grid(const ntc_material& M, int j, int k,
     const int bits = k ? M.bits1 : M.bits0;
     const float off = level_offset(bits);
     const int cb = cell_bytes(c, bits);
-    const uint8_t* base = static_cast<const uint8_t*>(k ? L.grid1 : L.grid0);
     Cell cl[4];
 #pragma unroll
-    for (int tp = 0; tp < 4; ++tp) cl[tp] = load_cell(base, t.cell[tp], cb);
+    for (int tp = 0; tp < 4; ++tp) cl[tp] = load_cell(static_cast<const uint8_t*>(base), t.cell[tp], cb);
+#pragma unroll 1
+    for (int ch = 0; ch < c; ch += 4) {
+      // the four channels' 4 x bits bits lie in one 64-bit half of the cell
+      const int bit = ch * bits;
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int c4 = 0; c4 < kMaxGridCh / 4; ++c4)
-      if (4 * c4 < c) {
+      for (int tp = 0; tp < 4; ++tp) {
+        uint32_t w = (uint32_t)((bit < 64 ? cl[tp].lo : cl[tp].hi) >> (bit & 63));
 #pragma unroll
-        for (int tp = 0; tp < 4; ++tp)
-#pragma unroll
-          for (int ch = 4 * c4; ch < 4 * c4 + 4; ++ch)
-            if (ch < c)
-              gs.acc[ch] = fmaf(t.w[tp], level_value(cell_index(cl[tp], ch, bits), off, q), gs.acc[ch]);
+        for (int i = 0; i < 4; ++i) {
+          v[i] = fmaf(t.w[tp], level_value(w & ((1u << bits) - 1u), off, q), v[i]);
+          w >>= bits;
+        }
       }
-  } else {
-    const float* base = static_cast<const float*>(k ? L.grid1 : L.grid0);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (ch + i >= c) v[i] = 0.f;
+      out(ch, v);
+    }
+    return;
+  }
+  // FP32 values, the next quad's loads in flight while this one is blended
+  const float* g = static_cast<const float*>(base);
+  const bool quads = (c & 3) == 0;
+  auto load = [&](int ch, float (&e)[4][4]) {
 #pragma unroll
     for (int tp = 0; tp < 4; ++tp) {
-      const float* g = base + (size_t)t.cell[tp] * c;
-      if ((c & 3) == 0) {
-#pragma unroll
-        for (int c4 = 0; c4 < kMaxGridCh / 4; ++c4)
-          if (4 * c4 < c) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(g) + c4);
-            float e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              float val = e[i];
-              if (noise) val += noise_of(nkey, j, k, t.cell[tp], 4 * c4 + i, c, q);
-              gs.acc[4 * c4 + i] = fmaf(t.w[tp], val, gs.acc[4 * c4 + i]);
-            }
-          }
+      const float* p = g + (size_t)t.cell[tp] * c + ch;
+      if (quads) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+        e[tp][0] = f.x; e[tp][1] = f.y; e[tp][2] = f.z; e[tp][3] = f.w;
       } else {
 #pragma unroll
-        for (int ch = 0; ch < kMaxGridCh; ++ch)
-          if (ch < c) {
-            float val = __ldg(g + ch);
-            if (noise) val += noise_of(nkey, j, k, t.cell[tp], ch, c, q);
-            gs.acc[ch] = fmaf(t.w[tp], val, gs.acc[ch]);
-          }
+        for (int i = 0; i < 4; ++i) e[tp][i] = ch + i < c ? __ldg(p + i) : 0.f;
       }
     }
+  };
+  float nx[4][4];
+  load(0, nx);
+#pragma unroll 1
+  for (int ch = 0; ch < c; ch += 4) {
+    float e[4][4];
+#pragma unroll
+    for (int tp = 0; tp < 4; ++tp)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) e[tp][i] = nx[tp][i];
+    if (ch + 4 < c) load(ch + 4, nx);
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int tp = 0; tp < 4; ++tp) {
+      if (noise) {
+        const float2 n0 = noise_pair(nkey, j, k, t.cell[tp], ch, c, q);
+        const float2 n1 = noise_pair(nkey, j, k, t.cell[tp], ch + 2, c, q);
+        e[tp][0] += n0.x; e[tp][1] += n0.y; e[tp][2] += n1.x; e[tp][3] += n1.y;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = fmaf(t.w[tp], e[tp][i], v[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (ch + i >= c) v[i] = 0.f;
+    out(ch, v);
   }
 }
 
@@ -353,22 +380,26 @@ __device__ __forceinline__ void grid_features(const ntc_material& M, int k, int 
       for (int tp = 0; tp < 4; ++tp) cl[tp] = load_cell(static_cast<const uint8_t*>(L.grid0), t.cell[tp], cb);
 #pragma unroll
       for (int tp = 0; tp < 4; ++tp)
+#pragma unroll 1
         for (int ch = 0; ch < M.c0; ++ch)
           sink(tp * M.c0 + ch, level_value(cell_index(cl[tp], ch, M.bits0), off, M.q0));
     } else {
 #pragma unroll 1
       for (int tp = 0; tp < 4; ++tp)
+#pragma unroll 1
         for (int ch = 0; ch < M.c0; ++ch)
           sink(tp * M.c0 + ch, grid_value(M, j, 0, t.cell[tp], ch, noise, nkey));
     }
     return;
   }
-  GridSample gs;
-  sample_grid(M, j, k, x, y, wm, hm, noise, nkey, gs);
+  const ntc_level& L = M.lv[j];
   const int c = k ? M.c1 : M.c0, s0 = k ? (learned ? 4 * M.c0 : M.c0) : 0;
+  const Taps t = bilinear_taps(x, y, wm, hm, k ? L.g1_w : L.g0_w, k ? L.g1_h : L.g0_h);
+  grid_quads<false>(M, j, k, t, noise, nkey, [&](int ch, const float (&v)[4]) {
 #pragma unroll
-  for (int ch = 0; ch < kMaxGridCh; ++ch)
-    if (ch < c) sink(s0 + ch, gs.acc[ch]);
+    for (int i = 0; i < 4; ++i)
+      if (ch + i < c) sink(s0 + ch + i, v[i]);
+  });
 }
 
 // The slots after the grids: 12 positional-encoding values, m/(M-1), zeros.
@@ -386,8 +417,8 @@ __device__ __forceinline__ void tail_features(const ntc_material& M, int x, int 
 template <class Sink>
 __device__ __forceinline__ void featurize(const ntc_material& M, int x, int y, int m, bool noise,
                                           uint64_t nkey, Sink& sink) {
-  grid_features(M, 0, x, y, m, noise, nkey, sink);
-  grid_features(M, 1, x, y, m, noise, nkey, sink);
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) grid_features(M, k, x, y, m, noise, nkey, sink);
   tail_features(M, x, y, m, sink);
 }
 

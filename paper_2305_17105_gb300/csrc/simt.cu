@@ -77,6 +77,7 @@ __device__ __forceinline__ float4 weight4(const ntc_material& M, const void* w, 
 template <class Place>
 __device__ __forceinline__ void stage_hidden(const ntc_material& M, const void* w, float scale,
                                              int ld, float* dst, Place place) {
+#pragma unroll 4
   for (int i = threadIdx.x; i < kHidden * (ld / 4); i += blockDim.x) {
     const int o = i & (kHidden - 1), k = 4 * (i >> 6);
     const float4 v = weight4(M, w, scale, o * ld + k);
@@ -159,13 +160,16 @@ __device__ __forceinline__ void warp_dense(const float* __restrict__ W, const fl
 __device__ __forceinline__ void put_hidden(float* act, int lane, int fn, float2 (&z)[8][4]) {
   __syncwarp();
   float* p = act + (lane & 7) * kLd + 4 * (lane >> 3);
+  auto apply = [&](int f) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) z[j][i] = make_float2(act_fwd(f, z[j][i].x), act_fwd(f, z[j][i].y));
+  };
+  if (fn == NTC_ACT_RELU) apply(NTC_ACT_RELU);
+  else apply(NTC_ACT_HARDGELU);
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      z[j][i].x = act_fwd(fn, z[j][i].x);
-      z[j][i].y = act_fwd(fn, z[j][i].y);
-    }
     *reinterpret_cast<float4*>(p + 8 * j * kLd) = make_float4(z[j][0].x, z[j][0].y, z[j][1].x, z[j][1].y);
     *reinterpret_cast<float4*>(p + 8 * j * kLd + 16) = make_float4(z[j][2].x, z[j][2].y, z[j][3].x, z[j][3].y);
   }
@@ -235,14 +239,13 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) decode_simt_kernel(
       }
       featurize(M, x, yy, m, noise != 0, nkey, sink);
       __syncwarp();
-      float2 z[8][4];
-      warp_dense<8>(smem + L.w1, smem + L.b1, act, K, lane, z);
-      put_hidden(act, lane, M.act, z);
-      warp_dense<8>(smem + L.w2, smem + L.b2, act, kHidden, lane, z);
-      put_hidden(act, lane, M.act, z);
-      if (L.h3) {
-        // third hidden layer (Sec. 4.4: activations on three layers)
-        warp_dense<8>(smem + L.wh, smem + L.bh, act, kHidden, lane, z);
+      // the hidden layers (two, or three: Sec. 4.4), one body
+#pragma unroll 1
+      for (int l = 0; l < (L.h3 ? 3 : 2); ++l) {
+        const float* w = smem + (l == 0 ? L.w1 : (l == 1 ? L.w2 : L.wh));
+        const float* b = smem + (l == 0 ? L.b1 : (l == 1 ? L.b2 : L.bh));
+        float2 z[8][4];
+        warp_dense<8>(w, b, act, l == 0 ? K : kHidden, lane, z);
         put_hidden(act, lane, M.act, z);
       }
       float2 o[2][4];
@@ -387,20 +390,17 @@ struct SB {
 
 __device__ __forceinline__ int place16(int n) { return 4 * (n & 15) + (n >> 4); }
 
-// Row-major W [rows][ld] -> [row][64] with column i at place16(i): the
-// backward's operand (lanes take consecutive columns: different banks).
-__device__ __forceinline__ void stage_backward(const ntc_material& M, const void* w, float scale,
-                                               int rows, int ld, int live, float* dst) {
-  for (int i = threadIdx.x; i < rows * kHidden; i += blockDim.x) {
-    const int o = i >> 6, k = i & (kHidden - 1);
-    float v = 0.f;
-    if (o < live && k < ld) {
-      const int e = o * ld + k;
-      if (M.precision == NTC_PREC_F16) v = __half2float(static_cast<const __half*>(w)[e]);
-      else if (M.precision == NTC_PREC_F8) v = (float)static_cast<const __nv_fp8_e4m3*>(w)[e] * scale;
-      else v = __ldg(static_cast<const float*>(w) + e);
-    }
-    dst[o * kHidden + place16(k)] = v;
+// The backward's operand of a hidden layer, [64 o][64] with column k at
+// place16(k) (zero from `cols` on), from the forward's [k][64] with output o
+// at place16(o).  Lane l of step d moves (o, k) = (l, (l + d) mod 32) of a
+// 32 x 32 block, so both sides hit 32 different banks.
+__device__ __forceinline__ void transpose_hidden(const float* __restrict__ f, int cols,
+                                                 float* __restrict__ dst) {
+  const int l = threadIdx.x & 31;
+#pragma unroll 4
+  for (int i = threadIdx.x >> 5; i < 4 * 32; i += kBThreads / 32) {
+    const int o = 32 * (i >> 6) + l, k = 32 * ((i >> 5) & 1) + ((l + i) & 31);
+    dst[o * kHidden + place16(k)] = k < cols ? f[k * kHidden + place16(o)] : 0.f;
   }
 }
 
@@ -431,13 +431,17 @@ __device__ __forceinline__ void put_units(float* dst, int ng, int qg, const floa
 }
 // z -> act(z), keeping act'(z).
 __device__ __forceinline__ void activate(int fn, float2 (&z)[4][2], float2 (&g)[4][2]) {
+  auto apply = [&](int f) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      g[j][p] = make_float2(act_grad(fn, z[j][p].x), act_grad(fn, z[j][p].y));
-      z[j][p] = make_float2(act_fwd(fn, z[j][p].x), act_fwd(fn, z[j][p].y));
-    }
+      for (int p = 0; p < 2; ++p) {
+        g[j][p] = make_float2(act_grad(f, z[j][p].x), act_grad(f, z[j][p].y));
+        z[j][p] = make_float2(act_fwd(f, z[j][p].x), act_fwd(f, z[j][p].y));
+      }
+  };
+  if (fn == NTC_ACT_RELU) apply(NTC_ACT_RELU);
+  else apply(NTC_ACT_HARDGELU);
 }
 
 // acc[r][s] += sum over the 32 texels of d[og + 16 r] h[ig + 8 s] (rows of
@@ -512,14 +516,17 @@ __global__ void __launch_bounds__(kBThreads, 2) backward_simt_kernel(const ntc_m
       d[2 * kMaxC] = v.z;
       d[3 * kMaxC] = v.w;
     }
-    stage_backward(M, M.w[0], s1, kHidden, K, kHidden, smem + S.w1b);
-    stage_backward(M, M.w[1], s2, kHidden, kHidden, kHidden, smem + S.w2b);
-    stage_backward(M, M.w[2], s3, kMaxC, kHidden, C, smem + S.w3b);
     for (int i = tid; i < kHidden; i += kBThreads) {
       smem[S.b1 + i] = M.b[0][i];
       smem[S.b2 + i] = M.b[1][i];
     }
     if (tid < kMaxC) smem[S.b3 + tid] = tid < C ? M.b[2][tid] : 0.f;
+    __syncthreads();
+    transpose_hidden(smem + S.w1f, K, smem + S.w1b);
+    transpose_hidden(smem + S.w2f, kHidden, smem + S.w2b);
+#pragma unroll 4
+    for (int i = tid; i < kMaxC * kHidden; i += kBThreads)
+      smem[S.w3b + (i >> 6) * kHidden + place16(i & 63)] = smem[S.w3f + (i & 63) * kMaxC + (i >> 6)];
   }
   const int64_t step = A.step_dev ? *A.step_dev : A.noise_step;
   const uint64_t nkey = rng_key(A.noise_seed, noise_stream(step));

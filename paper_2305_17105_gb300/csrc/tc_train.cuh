@@ -435,7 +435,7 @@ __device__ __forceinline__ void ld_nc_v8(const float* p, float4& a, float4& b) {
 
 // Channels 8 g .. 8 g + 7 (those below c; the others are zero) of the bilinear
 // sample of one FP32 grid of c = 4k <= 16 channels at `base`: all taps' loads
-// issued before the interpolation (same FMA order as sample_grid, so the same
+// issued before the interpolation (same FMA order as grid_quads, so the same
 // values); 32-byte loads where every group is whole and aligned (one L1
 // wavefront brings 8 channels).
 __device__ __forceinline__ void sample_group_f32(const float* base, int c, const Taps& t, int g,
@@ -963,17 +963,26 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
               else put_x(W, P, row, s0 + g, v);
             }
         } else {
-          GridSample gs;
-          sample_grid<true>(M, j, k, x, y, wm, hm, noise_on && valid, nkey, gs);
+          // (noise per tap, odd or wide grids: four channels at a time, in
+          // groups of eight with zeros behind the last channel)
+          const ntc_level& L = M.lv[j];
+          const Taps t = bilinear_taps(x, y, wm, hm, k ? L.g1_w : L.g0_w, k ? L.g1_h : L.g0_h);
+          float lo[4] = {0.f, 0.f, 0.f, 0.f};
+          auto put = [&](int ch, const float (&q)[4], bool last) {
+            float v[8];
 #pragma unroll
-          for (int g = 0; g < kGridPad / 8; ++g)
-            if (g < ng) {
-              float v[8];
-#pragma unroll
-              for (int e = 0; e < 8; ++e) v[e] = valid ? gs.acc[8 * g + e] : 0.f;
-              if (F8) put_x8(W, P, row, s0 + g, v, 1.f / sa[0], false, am[0]);
-              else put_x(W, P, row, s0 + g, v);
+            for (int e = 0; e < 4; ++e) {
+              const float f = valid ? q[e] : 0.f;
+              v[e] = (ch & 4) ? lo[e] : f;
+              v[4 + e] = (ch & 4) ? f : 0.f;
+              lo[e] = f;
             }
+            if ((ch & 4) == 0 && !last) return;
+            if (F8) put_x8(W, P, row, s0 + (ch >> 3), v, 1.f / sa[0], false, am[0]);
+            else put_x(W, P, row, s0 + (ch >> 3), v);
+          };
+          grid_quads<true>(M, j, k, t, noise_on && valid, nkey,
+                           [&](int ch, const float (&q)[4]) { put(ch, q, ch + 4 >= ck); });
         }
       };
       if (LEARNED) {
