@@ -1054,7 +1054,7 @@ int ntc_train_step_batched(const ntc_train_batch* batch, void* stream) {
   cls.hidden_layers = batch->hidden_layers;
   cls.precision = NTC_PREC_F16;
   e = ntc::launch_train_tc_batched(dev, cls, batch->total_tiles, batch->k_layout,
-                                   batch->dx_layout, (batch->flags & NTC_FLAG_CROPS) != 0, s);
+                                   batch->dx_layout, s);
   if (e != cudaSuccess) return cuda_status(e, "train batch: forward/backward");
   if (batch->flags & NTC_FLAG_GRAD_ONLY) return NTC_OK;
   return cuda_status(ntc::launch_adam_batched(dev, batch->adam_blocks, s), "train batch: adam");

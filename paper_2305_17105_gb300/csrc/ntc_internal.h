@@ -180,8 +180,7 @@ struct TrainBatchDev {
 // act, interp0 and hidden_layers (the kernel class) and the layout of the
 // largest k_int / dX width.
 cudaError_t launch_train_tc_batched(const TrainBatchDev* dev, const ntc_material& first,
-                                    int64_t total_tiles, int k_lay, int dx_lay, int crops,
-                                    cudaStream_t s);
+                                    int64_t total_tiles, int k_lay, int dx_lay, cudaStream_t s);
 // Pipelines per CTA of the batched step for that class and layout (0: none fits).
 int train_pipelines_layout(const ntc_material& first, int k_lay, int dx_lay);
 // Internal widths of a material's training rows: k_int and the dX columns.

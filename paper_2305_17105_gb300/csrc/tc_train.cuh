@@ -163,6 +163,11 @@ struct TPlan {
 struct MipTabT {
   int wm[16], hm[16], level[16];
   float lodn[16];
+  // the encoding's values are exact in FP16 and depend on c & 7 alone: per
+  // coordinate the (sin, cos) pairs of three octaves; the LOD input's FP16
+  // head and tail
+  uint32_t lodh[16], lodt[16];
+  uint4 pe[8];
 };
 
 // User column of internal input slot s: >= 0 a W1 column, -1 zero padding,
@@ -356,7 +361,22 @@ __device__ void stage_train(const ntc_material& M, const TPlan& P, uint8_t* sm) 
     tb->wm[m] = mip_dim(M.width, m);
     tb->hm[m] = mip_dim(M.height, m);
     tb->level[m] = level_of_mip(m, M.levels);
-    tb->lodn[m] = M.mips > 1 ? (float)m / (float)(M.mips - 1) : 0.f;
+    const float lod = M.mips > 1 ? (float)m / (float)(M.mips - 1) : 0.f;
+    tb->lodn[m] = lod;
+    tb->lodh[m] = tc::pack_f16x2(lod, 0.f);
+    tb->lodt[m] = tc::pack_f16x2(lod - __half2float(__float2half_rn(lod)), 0.f);
+  }
+  {
+    struct Pe {
+      float v[16];
+      __device__ void operator()(int i, float t) { v[i] = t; }
+    };
+    for (int c = tid; c < 8; c += nt) {
+      Pe pe;
+      positional_encoding(c, 0, 0, pe);
+      tb->pe[c] = make_uint4(tc::pack_f16x2(pe.v[0], pe.v[1]), tc::pack_f16x2(pe.v[2], pe.v[3]),
+                             tc::pack_f16x2(pe.v[4], pe.v[5]), 0u);
+    }
   }
   // the constant-one tiles of every pipeline: columns 0 and 1 are one
   // (ONEa, ONEc: groups 0 and 1; ONEb: group 0)
@@ -607,6 +627,20 @@ __device__ __forceinline__ void hidden_backward(uint32_t taddr, const uint8_t* g
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
       const uint32_t u[4] = {hw[g].x, hw[g].y, hw[g].z, hw[g].w};
+      if (ACT == NTC_ACT_RELU && !F8) {
+        // the rounded pair, cleared where H is not positive
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          union { uint32_t u; __half2 h; } c;
+          c.u = u[j];
+          w[j] = tc::pack_f16x2(a[8 * g + 2 * j], a[8 * g + 2 * j + 1]) &
+                 __hgt2_mask(c.h, __float2half2_rn(0.f));
+        }
+        *reinterpret_cast<uint4*>(htile + tc::canon_chunk(row, 4 * half + 2 * q + g, kRows)) =
+            make_uint4(w[0], w[1], w[2], w[3]);
+        continue;
+      }
       float v[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
@@ -993,23 +1027,33 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
         grid_rows(hf);
       }
       if (hf) {
-      struct Pe {
-        float v[16];
-        __device__ void operator()(int q, float t) { v[q] = t; }
-      } pe;
-      positional_encoding(x, y, 0, pe);
-      float v[8];
+      if (F8) {
+        struct Pe {
+          float v[16];
+          __device__ void operator()(int q, float t) { v[q] = t; }
+        } pe;
+        positional_encoding(x, y, 0, pe);
+        float v[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = pe.v[e];
-      if (F8) put_x8(W, P, row, P.gpe, v, 1.f / sa[0], false, am[0]);
-      else put_x(W, P, row, P.gpe, v);
+        for (int e = 0; e < 8; ++e) v[e] = pe.v[e];
+        put_x8(W, P, row, P.gpe, v, 1.f / sa[0], false, am[0]);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = pe.v[8 + e];
-      v[4] = tb->lodn[m];
-      v[5] = 0.f;
-      v[6] = v[7] = 1.f;
-      if (F8) put_x8(W, P, row, P.gpe + 1, v, 1.f / sa[0], true, am[0]);
-      else put_x(W, P, row, P.gpe + 1, v);
+        for (int e = 0; e < 4; ++e) v[e] = pe.v[8 + e];
+        v[4] = tb->lodn[m];
+        v[5] = 0.f;
+        v[6] = v[7] = 1.f;
+        put_x8(W, P, row, P.gpe + 1, v, 1.f / sa[0], true, am[0]);
+      } else {
+        const uint4 px = tb->pe[x & 7], py = tb->pe[y & 7];
+        const uint32_t o = tc::canon_chunk(row, 0, kRows);
+        auto put = [&](int g, uint4 head, uint4 tail) {
+          *reinterpret_cast<uint4*>(W + P.X + (uint32_t)g * kGroup + o) = head;
+          *reinterpret_cast<uint4*>(W + xlo_group(P, g) + o) = tail;
+        };
+        put(P.gpe, make_uint4(px.x, px.y, px.z, py.x), make_uint4(0, 0, 0, 0));
+        put(P.gpe + 1, make_uint4(py.y, py.z, tb->lodh[m], tc::pack_f16x2(1.f, 1.f)),
+            make_uint4(0, 0, tb->lodt[m], 0));
+      }
       const float zz[8] = {0, 0, 0, 0, 0, 0, 0, 0};
       for (int g = P.gpe + 2; g < P.k_int / 8; ++g) {
         if (F8) put_x8(W, P, row, g, zz, 1.f, false, am[0]);
@@ -1519,17 +1563,15 @@ int pipelines_for(const ntc_material& m, int k_lay, int dx_lay) {
 }
 int train_pipelines(const ntc_material& m) { return pipelines_for(m, 0, 0); }
 
-// Pipelines per CTA: the autotuner's choice (a.pipelines), else by the call.
-// Independent texels: two (their random gathers and reductions want the L1
-// that a third pipeline's tiles take, and 128 registers a thread: 2^18 texels
-// of a 2048^2 x 12 material 104 us against 112 with three); crops, whose
-// neighbours share cells: three where they fit (83 -> 79 us); a call with no
-// more tiles than SMs: one.
+// Pipelines per CTA: the autotuner's choice (a.pipelines), else two (a third
+// would leave 80 registers a thread and take L1 from the gathers: 2^18 texels
+// of a 2048^2 x 12 material 102 us against 115 with three, as crops 80
+// against 81), or one for a call with no more tiles than SMs.
 template <int ACT, bool LEARNED, bool BATCHED, bool F8>
 cudaError_t launch_n(const ntc_material& m, const BwdArgs& a, const TrainBatchDev* hb,
                      int64_t tiles, int k_lay, int dx_lay, cudaStream_t s) {
   const int most = pipelines_for(m, k_lay, dx_lay);
-  const int want = a.pipelines > 0 ? a.pipelines : (tiles <= sm_count() ? 1 : (a.crops ? 3 : 2));
+  const int want = a.pipelines > 0 ? a.pipelines : (tiles <= sm_count() ? 1 : 2);
   const int np = want < most ? want : most;
   switch (np) {
     case 3: return launch_t<ACT, LEARNED, 3, BATCHED, F8>(m, a, hb, tiles, k_lay, dx_lay, s);

@@ -6,13 +6,10 @@
 namespace ntc {
 
 cudaError_t launch_train_tc_batched(const TrainBatchDev* dev, const ntc_material& first,
-                                    int64_t total_tiles, int k_lay, int dx_lay, int crops,
-                                    cudaStream_t s) {
+                                    int64_t total_tiles, int k_lay, int dx_lay, cudaStream_t s) {
   if (total_tiles == 0) return cudaSuccess;
   if (pipelines_for(first, k_lay, dx_lay) == 0) return cudaErrorNotSupported;
-  BwdArgs a{};  // each material's arguments are in `dev`; these choose the pipelines
-  a.crops = crops;
-  return launch_class<true>(first, a, dev, total_tiles, k_lay, dx_lay, s);
+  return launch_class<true>(first, BwdArgs{}, dev, total_tiles, k_lay, dx_lay, s);
 }
 
 }  // namespace ntc
