@@ -8,9 +8,9 @@
 // epilogue each takes one half of the columns, in the scatter one half of the
 // warp's texels.  The step is bound by the latency of a tile's serial chain
 // (issue slots a fifth used).  With one thread a row and the MMAs issued by a
-// divergent thread a tile alone took 12.6 us, now 8.9; a step of 2^18 texels
-// of a 2048^2 x 12 material 176 -> 160 us, of eight crops on the paper's
-// decoder 353 -> 268 us.
+// divergent thread a tile alone took 12.6 us, now 8.6; a step of 2^18 texels
+// of a 2048^2 x 12 material 176 -> 154 us, of eight crops on the paper's
+// decoder 353 -> 259 us.
 // Per tile, with every activation kept on chip:
 //   forward   X -> Z1 = X W1^T (+b1) -> H1 = act(Z1) -> Z2 (+b2) -> H2 -> Z3 (+b3)
 //             -> y = out(Z3), loss, dZ3 = 2 (y - t) out'(Z3); with a third
@@ -1027,43 +1027,43 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
         grid_rows(hf);
       }
       if (hf) {
-      if (F8) {
-        struct Pe {
-          float v[16];
-          __device__ void operator()(int q, float t) { v[q] = t; }
-        } pe;
-        positional_encoding(x, y, 0, pe);
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = pe.v[e];
-        put_x8(W, P, row, P.gpe, v, 1.f / sa[0], false, am[0]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = pe.v[8 + e];
-        v[4] = tb->lodn[m];
-        v[5] = 0.f;
-        v[6] = v[7] = 1.f;
-        put_x8(W, P, row, P.gpe + 1, v, 1.f / sa[0], true, am[0]);
-      } else {
-        const uint4 px = tb->pe[x & 7], py = tb->pe[y & 7];
-        const uint32_t o = tc::canon_chunk(row, 0, kRows);
-        auto put = [&](int g, uint4 head, uint4 tail) {
-          *reinterpret_cast<uint4*>(W + P.X + (uint32_t)g * kGroup + o) = head;
-          *reinterpret_cast<uint4*>(W + xlo_group(P, g) + o) = tail;
-        };
-        put(P.gpe, make_uint4(px.x, px.y, px.z, py.x), make_uint4(0, 0, 0, 0));
-        put(P.gpe + 1, make_uint4(py.y, py.z, tb->lodh[m], tc::pack_f16x2(1.f, 1.f)),
-            make_uint4(0, 0, tb->lodt[m], 0));
-      }
-      const float zz[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (int g = P.gpe + 2; g < P.k_int / 8; ++g) {
-        if (F8) put_x8(W, P, row, g, zz, 1.f, false, am[0]);
-        else put_x(W, P, row, g, zz);
-      }
-      // the E4M3 tile's K padding up to a multiple of 32 inputs
-      if (F8)
-        for (int g = P.k_int / 8; g < P.k8 / 8; ++g)
-          *reinterpret_cast<uint2*>(W + P.H1 + tc::canon_chunk(row, g >> 1, kRows) + (g & 1) * 8) =
-              make_uint2(0u, 0u);
+        if (F8) {
+          struct Pe {
+            float v[16];
+            __device__ void operator()(int q, float t) { v[q] = t; }
+          } pe;
+          positional_encoding(x, y, 0, pe);
+          float v[8];
+  #pragma unroll
+          for (int e = 0; e < 8; ++e) v[e] = pe.v[e];
+          put_x8(W, P, row, P.gpe, v, 1.f / sa[0], false, am[0]);
+  #pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = pe.v[8 + e];
+          v[4] = tb->lodn[m];
+          v[5] = 0.f;
+          v[6] = v[7] = 1.f;
+          put_x8(W, P, row, P.gpe + 1, v, 1.f / sa[0], true, am[0]);
+        } else {
+          const uint4 px = tb->pe[x & 7], py = tb->pe[y & 7];
+          const uint32_t o = tc::canon_chunk(row, 0, kRows);
+          auto put = [&](int g, uint4 head, uint4 tail) {
+            *reinterpret_cast<uint4*>(W + P.X + (uint32_t)g * kGroup + o) = head;
+            *reinterpret_cast<uint4*>(W + xlo_group(P, g) + o) = tail;
+          };
+          put(P.gpe, make_uint4(px.x, px.y, px.z, py.x), make_uint4(0, 0, 0, 0));
+          put(P.gpe + 1, make_uint4(py.y, py.z, tb->lodh[m], tc::pack_f16x2(1.f, 1.f)),
+              make_uint4(0, 0, tb->lodt[m], 0));
+        }
+        const float zz[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        for (int g = P.gpe + 2; g < P.k_int / 8; ++g) {
+          if (F8) put_x8(W, P, row, g, zz, 1.f, false, am[0]);
+          else put_x(W, P, row, g, zz);
+        }
+        // the E4M3 tile's K padding up to a multiple of 32 inputs
+        if (F8)
+          for (int g = P.k_int / 8; g < P.k8 / 8; ++g)
+            *reinterpret_cast<uint2*>(W + P.H1 + tc::canon_chunk(row, g >> 1, kRows) + (g & 1) * 8) =
+                make_uint2(0u, 0u);
       }
     }
     tc::fence_proxy_async();
@@ -1157,26 +1157,34 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
 #pragma unroll
         for (int c = 0; c < 8; ++c) zv[c] = fmaf(zv[c], sa[2] * sw[2], b3[c]);
       }
+      // dY from the target texel (loss mode) or the upstream gradient row (dout
+      // mode), without a branch per channel
+      const bool ident = M.out_act == NTC_OUT_IDENTITY;
+      const int live = valid ? C - 8 * hf : 0;  // channels of this half that count
+      float yc[8], dy[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        // sigmoid; the fast division is within 2 ulp
+        const float sg = __fdividef(1.f, 1.f + __expf(-zv[c]));
+        yc[c] = ident ? zv[c] : sg;
+      }
+      if (A.target) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float t = (float)((tw[c >> 2] >> (8 * (c & 3))) & 0xFFu) * (1.f / 255.f);
+          const float e = c < live ? yc[c] - t : 0.f;
+          loss_acc = fmaf(e, e, loss_acc);
+          dy[c] = 2.f * e;
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) dy[c] = c < live ? A.dout[i * C + 8 * hf + c] * dscale : 0.f;
+      }
       float v[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        float g = 0.f;
-        if (valid && 8 * hf + c < C) {
-          // the target texel (loss mode) or the upstream gradient row (dout mode)
-          const float tgt = A.target ? (float)((tw[c >> 2] >> (8 * (c & 3))) & 0xFFu) * (1.f / 255.f)
-                                     : A.dout[i * C + 8 * hf + c];
-          // sigmoid; the fast division is within 2 ulp
-          const float yc = M.out_act == NTC_OUT_IDENTITY ? zv[c] : __fdividef(1.f, 1.f + __expf(-zv[c]));
-          if (A.target) {
-            const float e = yc - tgt;
-            loss_acc = fmaf(e, e, loss_acc);
-            g = M.out_act == NTC_OUT_IDENTITY ? 2.f * e : 2.f * e * yc * (1.f - yc);
-          } else {
-            const float d = tgt * dscale;
-            g = M.out_act == NTC_OUT_IDENTITY ? d : d * yc * (1.f - yc);
-          }
-        }
-        v[c] = g;
+        const float g = ident ? dy[c] : dy[c] * yc[c] * (1.f - yc[c]);
+        v[c] = c < live ? g : 0.f;
       }
       put_chunk(W + P.DZ3, row, hf, v);
     }
