@@ -22,8 +22,8 @@ namespace {
 // What bounds it: the FP32 FMA rate (78.4 TFLOP/s measured).  One thread per
 // query with every weight broadcast from shared memory (the form this
 // replaced) needed a 16-byte load per four FMAs and was bound by them:
-// a pass of 65,536 queries of a 256^2 x 8 material took 86 us against 31 now
-// (25 of them the host's share of a call).
+// a pass of 65,536 queries of a 256^2 x 8 material took 86 us against 29 now
+// (22 of them the host's share of a call).
 // ---------------------------------------------------------------------------
 constexpr int kLd = 36;         // floats per unit row: 32 queries + 4 of padding
 constexpr int kMaxWarps = 16;   // tiles in flight per CTA (one CTA per SM)
@@ -360,7 +360,7 @@ __global__ void f8_scales_kernel(const uint32_t* amax, float* sa) {
 // one tile, hence small tiles spread over all SMs, with the rows' features
 // split over the warps (G0, G1, the encoding and target, the taps).  Tiles
 // of 128 texels, one per thread, ran a 4,096-texel step of a 256^2 x 8
-// material on 32 CTAs in 118 us (all launches of the step) against 47 now.
+// material on 32 CTAs in 118 us (all launches of the step) against 39 now.
 // ---------------------------------------------------------------------------
 constexpr int kBTile = 32;
 constexpr int kBThreads = 128;

@@ -112,8 +112,9 @@ __device__ __forceinline__ void hidden_epilogue_q8(uint32_t td, uint32_t ta, int
 // by the row's thread (kWsPlain) or, for channel counts that are not multiples
 // of four, through shared memory (kWsRows); trilinear (kWsTri) or stochastic
 // filtering (kWsStoch).  Each is a kernel of its own: with the filter read at
-// run time the nearest decode's loop spilled (2^24 queries 531 -> 581 us).  NC: compute warpgroups, 5 for the layouts known at
-// compile time and the lattice form, 4 for those read from the plan.
+// run time the nearest decode's loop spilled (2^24 queries 531 -> 581 us).  NC:
+// compute warpgroups, 5 for the layouts known at compile time and the lattice
+// form, 4 for those read from the plan.
 template <int CLS, bool F8, bool H3, int MODE, int NC>
 __global__ void __launch_bounds__(ws_threads(NC), 1) decode_ws_kernel(
     const ntc_material M, const float* __restrict__ uvl, int64_t n, void* __restrict__ out,

@@ -1,16 +1,16 @@
 // Tensor-core (tcgen05) fused forward + L2 loss + backward of the NTC
 // optimisation step (Sec. 4.2, 4.5, 5.1), FP16 operands, FP32 accumulation.
 //
-// One persistent CTA per SM runs NWG pipelines (3, 2 or 1: the most whose
-// tiles fit in shared memory); a pipeline of 256 threads owns a stream of
-// tiles of 128 training texels (one row = one TMEM lane each).  Two threads
-// share a row: half 0 gathers G0, half 1 G1 and the encoding; in every
-// epilogue each takes one half of the columns, in the scatter one half of the
-// warp's texels.  The step is bound by the latency of a tile's serial chain
-// (issue slots a fifth used).  With one thread a row and the MMAs issued by a
-// divergent thread a tile alone took 12.6 us, now 8.6; a step of 2^18 texels
-// of a 2048^2 x 12 material 176 -> 154 us, of eight crops on the paper's
-// decoder 353 -> 259 us.
+// One persistent CTA per SM runs NWG pipelines (two, one for calls with no
+// more tiles than SMs, up to three on request, as far as their tiles fit in
+// shared memory); a pipeline of 256 threads owns a stream of tiles of 128
+// training texels (one row = one TMEM lane each).  Two threads share a row:
+// half 0 gathers G0, half 1 G1 and the encoding; in every epilogue each takes
+// one half of the columns, in the scatter one half of the warp's texels.  The
+// step is bound by the latency of a tile's serial chain (issue slots a quarter
+// used).  With one thread a row and the MMAs issued by a divergent thread a
+// tile alone took 12.6 us against 8.9; a step of 2^18 texels of a 2048^2 x 12
+// material 176 -> 154 us, of eight crops on the paper's decoder 353 -> 259 us.
 // Per tile, with every activation kept on chip:
 //   forward   X -> Z1 = X W1^T (+b1) -> H1 = act(Z1) -> Z2 (+b2) -> H2 -> Z3 (+b3)
 //             -> y = out(Z3), loss, dZ3 = 2 (y - t) out'(Z3); with a third
