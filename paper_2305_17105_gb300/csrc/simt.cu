@@ -3,6 +3,8 @@
 // optimisation (Sec. 4.3-4.5, 5.1, 5.3).  The MLP runs as register-tiled
 // FP32 matrix products on tiles of 32 queries / texels whose activations stay
 // in shared memory; every activation is recomputed on chip.
+#include <cooperative_groups.h>
+
 #include "ntc_device.cuh"
 #include "ntc_internal.h"
 
@@ -360,10 +362,11 @@ __global__ void f8_scales_kernel(const uint32_t* amax, float* sa) {
 // one tile, hence small tiles spread over all SMs, with the rows' features
 // split over the warps (G0, G1, the encoding and target, the taps).  Tiles
 // of 128 texels, one per thread, ran a 4,096-texel step of a 256^2 x 8
-// material on 32 CTAs in 118 us (all launches of the step) against 39 now.
+// material on 32 CTAs in 118 us (all launches of the step) against 36 now.
 // ---------------------------------------------------------------------------
 constexpr int kBTile = 32;
 constexpr int kBThreads = 128;
+constexpr int kBCluster = 4;   // CTAs that add their losses before one of them reduces
 constexpr int kTapMeta = 112;  // bytes per texel: 8 cell addresses, 8 weights, padding
 
 struct SB {
@@ -723,7 +726,20 @@ __global__ void __launch_bounds__(kBThreads, 2) backward_simt_kernel(const ntc_m
     float* red = smem + S.red;
     if (lane == 0) red[warp] = loss_acc;
     __syncthreads();
-    if (tid == 0) atomicAdd(A.loss, (red[0] + red[1] + red[2] + red[3]) * A.loss_scale);
+    // One reduction per cluster: its CTAs' sums meet in the first one, so that
+    // the running total is rounded once per 128 (64) texels, not once per 32.
+    __shared__ float part[kBCluster];
+    auto cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    if (tid == 0)
+      *cluster.map_shared_rank(part + cluster.block_rank(), 0) =
+          (red[0] + red[1] + red[2] + red[3]) * A.loss_scale;
+    cluster.sync();
+    if (tid == 0 && cluster.block_rank() == 0) {
+      float sum = part[0];
+      for (unsigned k = 1; k < cluster.num_blocks(); ++k) sum += part[k];
+      atomicAdd(A.loss, sum);
+    }
   }
 }
 
@@ -790,9 +806,22 @@ cudaError_t launch_backward_simt(const ntc_material& m, const BwdArgs& a, cudaSt
   if (e != cudaSuccess) return e;
   const int64_t tiles = (a.n + kBTile - 1) / kBTile;
   const int64_t cap = 2 * (int64_t)sm_count();
-  const int grid = (int)(tiles < cap ? tiles : cap);
-  backward_simt_kernel<<<grid, kBThreads, smem, s>>>(m, a);
-  return cudaGetLastError();
+  const int64_t grid = tiles < cap ? tiles : cap;
+  // With two CTAs per SM clusters of four no longer find room for the whole
+  // grid at once (2^18 texels 451 -> 749 us), clusters of two do.
+  const unsigned cl = grid <= sm_count() ? kBCluster : 2;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((grid + cl - 1) / cl * cl));
+  cfg.blockDim = dim3(kBThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, backward_simt_kernel, m, a);
 }
 
 }  // namespace ntc
