@@ -697,6 +697,10 @@ __global__ void __launch_bounds__(kBThreads, 2) backward_simt_kernel(const ntc_m
   }
 
   // ---- flush: the CTA's weight gradients row-major over the weights' place ------
+  // The grid is a whole number of clusters, so its last CTAs may have no tile:
+  // they come here straight from the transposes, whose writes the staging
+  // below runs over.
+  __syncthreads();
   const float gs = A.grad_scale;
   float* f1 = smem;                        // [64][K]
   float* f2 = f1 + kHidden * K;            // [64][64]
