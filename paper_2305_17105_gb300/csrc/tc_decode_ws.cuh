@@ -26,7 +26,10 @@ namespace {
 // and its epilogue leaves H in place in [0, 32) (a quarter of the columns is
 // read before its half is written); layer 2 accumulates into [32, 96), its
 // epilogue writes H over [0, 32) again; layer 3 accumulates into [80, 96),
-// clear of the next tile's layer 1.
+// clear of the next tile's layer 1.  That layer's accumulator covers the H
+// which layer 3 reads, and two MMAs are ordered by themselves only where they
+// share accumulator and shape: the issuer waits for layer 3's commit before
+// it issues the next layer 1.
 //
 // What bounds it: the latency of a tile's chain of stages, of which the warps
 // in flight hide part (issue slots half used, L1 three quarters).  96 columns
@@ -223,8 +226,9 @@ __global__ void __launch_bounds__(ws_threads(NC), 1) decode_ws_kernel(
       for (int tl = first; tl < ntiles; tl += stride) {
         asm volatile("" : "+r"(w2));  // form the descriptors below anew: hoisted, they would spill
         if (!(ok = wait_all(&bar_x[w], px))) break;
-        // trilinear: the previous tile's output has been read
-        if (tri && tl != first && !(ok = wait_all(&bar_r[w], px ^ 1))) break;
+        // the previous tile's layer 3 no longer reads H (trilinear: and its
+        // output has been read)
+        if (tl != first && !(ok = wait_all(tri ? &bar_r[w] : &bar_o[w], px ^ 1))) break;
         px ^= 1;
         tc::fence_after_sync();
         if (tc::elect_one()) {
