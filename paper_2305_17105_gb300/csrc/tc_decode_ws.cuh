@@ -459,10 +459,14 @@ inline int grid_class(int c, int cb) { return cb == 4 ? 0 : (c > 12 ? 2 : 1); }
 
 // Materials off the fast layout that take the lattice form: packed grids of 2
 // or 4 bits with the fast layout's exactness conditions (other widths, F32
-// grids and vector-quantised G0 blend in float).
+// grids and vector-quantised G0 blend in float), and a plan of which five
+// pipelines fit beside the kernel's own 1 KB.  It does not with learned G0,
+// three hidden layers and more than 16 channels in both grids (K = 144:
+// 232,448 bytes); the float form's four pipelines (195,584) do.
 inline bool lattice_ok(const ntc_material& m) {
   return m.encoding == NTC_GRID_PACKED && m.vq_books == 0 && (m.bits0 == 2 || m.bits0 == 4) &&
-         (m.bits1 == 2 || m.bits1 == 4) && fast_layout_ok(m);
+         (m.bits1 == 2 || m.bits1 == 4) && fast_layout_ok(m) &&
+         WsPlan(Plan(m, false, false), false, 5, m.channels, false).total <= 226u * 1024u;
 }
 
 // The FP16 form of one mode, by layout.
