@@ -257,7 +257,9 @@ cudaError_t launch_selftest_wait(uint32_t limit, cudaStream_t s) {
 
 // The fast layout's exactness conditions: every grid/mip size ratio of every
 // mip is a multiple of 1/8 (taps on the 1/16 lattice) and the bin widths are
-// powers of two in [2^-6, 2^6] (the half constants of ylerp_of exact).
+// powers of two in [2^-6, 2^6] (the half constants of ylerp_of exact).  A
+// learned G0's taps are dequantised as (1024 + k) Q - (1024 + off) Q in halves,
+// whose constant passes the largest half (65,504) at Q = 64.
 bool fast_layout_ok(const ntc_material& m) {
   for (int mi = 0; mi < m.mips; ++mi) {
     const int wm = mip_dim(m.width, mi), hm = mip_dim(m.height, mi);
@@ -269,6 +271,7 @@ bool fast_layout_ok(const ntc_material& m) {
     int e = 0;
     if (!(q > 0.f) || std::frexp(q, &e) != 0.5f || e < -5 || e > 7) return false;
   }
+  if (m.interp0 == NTC_INTERP_LEARNED && m.q0 > 32.f) return false;
   return true;
 }
 
