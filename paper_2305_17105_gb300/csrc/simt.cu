@@ -448,10 +448,13 @@ __device__ __forceinline__ void activate(int fn, float2 (&z)[4][2], float2 (&g)[
 }
 
 // acc[r][s] += sum over the 32 texels of d[og + 16 r] h[ig + 8 s] (rows of
-// units; s < cols / 8).
+// units; s < cols / 8).  The tile is summed by itself first: one chain over
+// all of a CTA's texels would round every product to the running total
+// (2^18 texels, K = 32: 2.8e-7 from 64 bits in dW1).
 template <int R>
 __device__ __forceinline__ void outer_acc(const float* __restrict__ d, const float* __restrict__ h,
                                           int og, int ig, int cols, float (&acc)[R][8]) {
+  float t[R][8] = {};
 #pragma unroll 1
   for (int q = 0; q < kBTile; q += 4) {
     float4 dv[R];
@@ -463,13 +466,17 @@ __device__ __forceinline__ void outer_acc(const float* __restrict__ d, const flo
         const float4 hv = *reinterpret_cast<const float4*>(h + (ig + 8 * s) * kLd + q);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          acc[r][s] = fmaf(dv[r].x, hv.x, acc[r][s]);
-          acc[r][s] = fmaf(dv[r].y, hv.y, acc[r][s]);
-          acc[r][s] = fmaf(dv[r].z, hv.z, acc[r][s]);
-          acc[r][s] = fmaf(dv[r].w, hv.w, acc[r][s]);
+          t[r][s] = fmaf(dv[r].x, hv.x, t[r][s]);
+          t[r][s] = fmaf(dv[r].y, hv.y, t[r][s]);
+          t[r][s] = fmaf(dv[r].z, hv.z, t[r][s]);
+          t[r][s] = fmaf(dv[r].w, hv.w, t[r][s]);
         }
       }
   }
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int s = 0; s < 8; ++s) acc[r][s] += t[r][s];
 }
 __device__ __forceinline__ float row_sum(const float* __restrict__ d) {
   float s = 0.f;
@@ -482,16 +489,25 @@ __device__ __forceinline__ float row_sum(const float* __restrict__ d) {
 }
 
 // The staged row-major array `src` (n floats, a multiple of 4) times `gs`
-// into the gradient at `g`.
-__device__ __forceinline__ void flush_rows(float* g, const float* src, int n, float gs) {
+// into the gradient at `g`.  With a `mate` (the same array of the other CTA of
+// a cluster of two) the sum of the two, each CTA every other block of the
+// elements.
+__device__ __forceinline__ void flush_rows(float* g, const float* src, const float* mate, int half,
+                                           int n, float gs) {
   if (!g) return;
+  const int first = threadIdx.x + (mate ? kBThreads * half : 0), step = mate ? 2 * kBThreads : kBThreads;
   if ((reinterpret_cast<uintptr_t>(g) & 15) == 0 && (n & 3) == 0) {
-    for (int i = threadIdx.x; i < n / 4; i += kBThreads) {
-      const float4 v = reinterpret_cast<const float4*>(src)[i];
+#pragma unroll 4
+    for (int i = first; i < n / 4; i += step) {
+      float4 v = reinterpret_cast<const float4*>(src)[i];
+      if (mate) {
+        const float4 o = reinterpret_cast<const float4*>(mate)[i];
+        v = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
+      }
       atomicAdd(reinterpret_cast<float4*>(g) + i, make_float4(v.x * gs, v.y * gs, v.z * gs, v.w * gs));
     }
   } else {
-    for (int i = threadIdx.x; i < n; i += kBThreads) atomicAdd(g + i, src[i] * gs);
+    for (int i = first; i < n; i += step) atomicAdd(g + i, (mate ? src[i] + mate[i] : src[i]) * gs);
   }
 }
 
@@ -717,34 +733,40 @@ __global__ void __launch_bounds__(kBThreads, 2) backward_simt_kernel(const ntc_m
   }
   fb[tid] = ab;
   if (tid < kMaxC) fb[2 * kHidden + tid] = ab3;
-  __syncthreads();
-  flush_rows(A.g.w[0], f1, kHidden * K, gs);
-  flush_rows(A.g.w[1], f2, kHidden * kHidden, gs);
-  flush_rows(A.g.w[2], f3, C * kHidden, gs);
-  flush_rows(A.g.b[0], fb, kHidden, gs);
-  flush_rows(A.g.b[1], fb + kHidden, kHidden, gs);
-  flush_rows(A.g.b[2], fb + 2 * kHidden, C, gs);
-  if (A.train && A.loss) {
+  const bool loss = A.train && A.loss;
+  if (loss) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
-    float* red = smem + S.red;
-    if (lane == 0) red[warp] = loss_acc;
-    __syncthreads();
-    // One reduction per cluster: its CTAs' sums meet in the first one, so that
-    // the running total is rounded once per 128 (64) texels, not once per 32.
-    __shared__ float part[kBCluster];
-    auto cluster = cooperative_groups::this_cluster();
-    cluster.sync();
-    if (tid == 0)
-      *cluster.map_shared_rank(part + cluster.block_rank(), 0) =
-          (red[0] + red[1] + red[2] + red[3]) * A.loss_scale;
-    cluster.sync();
-    if (tid == 0 && cluster.block_rank() == 0) {
-      float sum = part[0];
-      for (unsigned k = 1; k < cluster.num_blocks(); ++k) sum += part[k];
-      atomicAdd(A.loss, sum);
-    }
+    if (lane == 0) smem[S.red + warp] = loss_acc;
   }
+  // Two CTAs an SM come in clusters of two, which add their gradients before
+  // one reduction into memory: so many CTAs each round the running totals that
+  // with a reduction of each CTA's own the weight gradients of 2^15 to 2^18
+  // texels were 2.2e-7 to 3e-7 from 64 bits, against 1.6e-7 to 2.2e-7.
+  auto cluster = cooperative_groups::this_cluster();
+  const int rank = cluster.block_rank();
+  const bool pair = cluster.num_blocks() == 2;
+  if (pair) cluster.sync();
+  else __syncthreads();
+  const float* mate = pair ? cluster.map_shared_rank(smem, rank ^ 1) : nullptr;
+#pragma unroll 1
+  for (int l = 0; l < 6; ++l) {  // rolled: the code is fetched cold
+    float* g = l < 3 ? A.g.w[l] : A.g.b[l - 3];
+    const float* src = l == 0 ? f1 : (l == 1 ? f2 : (l == 2 ? f3 : fb + (l - 3) * kHidden));
+    const int n = l == 0 ? kHidden * K : (l == 1 ? kHidden * kHidden : (l == 2 ? C * kHidden : (l == 5 ? C : kHidden)));
+    flush_rows(g, src, pair ? mate + (src - smem) : nullptr, rank, n, gs);
+  }
+  if (loss && !pair) cluster.sync();
+  if (loss && tid == 0 && rank == 0) {
+    // the losses too: the running total is rounded once per 128 (64) texels
+    float sum = 0.f;
+    for (unsigned k = 0; k < cluster.num_blocks(); ++k) {
+      const float* red = cluster.map_shared_rank(smem + S.red, k);
+      sum += (red[0] + red[1] + red[2] + red[3]) * A.loss_scale;
+    }
+    atomicAdd(A.loss, sum);
+  }
+  if (pair || loss) cluster.sync();  // no CTA leaves while another reads its rows
 }
 
 }  // namespace
