@@ -813,10 +813,11 @@ __device__ __forceinline__ void join_runs(const uint8_t* at, Run r, int q) {
   if (r.cell) atomicAdd(reinterpret_cast<float4*>(r.cell) + q, r.acc);
 }
 
-// Wait for the pipeline's MMAs; after a wait that ran out (`bad`) no further
-// one is tried, and the pipeline leaves at the end of the tile.
+// Wait for the pipeline's MMAs.  A warp whose wait ran out (`bad`) touches no
+// operand or result of theirs any more; the pipeline leaves together at its
+// next barrier.
 __device__ __forceinline__ void wait_phase(uint64_t* bar, uint32_t& phase, bool& bad) {
-  if (!bad) bad = !tc::mbar_wait(bar, phase, kWaitLimit);
+  bad = __any_sync(0xffffffffu, !tc::mbar_wait(bar, phase, kWaitLimit));
   phase ^= 1;
 }
 
@@ -1115,15 +1116,17 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
       tc::mma_commit(bar);
     }
     wait_phase(bar, phase, bad);
-    tc::fence_after_sync();
-    if (F8)
-      hidden_forward_f8<ACT>(tD + lane, sa[0] * sw[0], reinterpret_cast<const float*>(sm + P.bf),
-                             1.f / sa[1], W + P.H1, W + P.H2, W + P.G1, row, hf, am[1]);
-    else
-      hidden_forward<ACT>(tD + lane, W + P.H1, W + P.G1, W + P.H2, row, hf);
-    tc::fence_before_sync();
-    tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kPipe);
+    if (!bad) {
+      tc::fence_after_sync();
+      if (F8)
+        hidden_forward_f8<ACT>(tD + lane, sa[0] * sw[0], reinterpret_cast<const float*>(sm + P.bf),
+                               1.f / sa[1], W + P.H1, W + P.H2, W + P.G1, row, hf, am[1]);
+      else
+        hidden_forward<ACT>(tD + lane, W + P.H1, W + P.G1, W + P.H2, row, hf);
+      tc::fence_before_sync();
+      tc::fence_proxy_async();
+    }
+    if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
 
     // ---- layer 2 -----------------------------------------------------------------
     if (pw == 0 && tc::elect_one()) {
@@ -1138,16 +1141,18 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
       tc::mma_commit(bar);
     }
     wait_phase(bar, phase, bad);
-    tc::fence_after_sync();
-    if (F8)
-      hidden_forward_f8<ACT>(tD + lane, sa[1] * sw[1],
-                             reinterpret_cast<const float*>(sm + P.bf) + kHidden, 1.f / sa[2],
-                             W + P.H2, W + P.S8, W + P.G2, row, hf, am[2]);
-    else
-      hidden_forward<ACT>(tD + lane, W + P.H2, W + P.G2, P.h3 ? W + P.H3 : nullptr, row, hf);
-    tc::fence_before_sync();
-    tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kPipe);
+    if (!bad) {
+      tc::fence_after_sync();
+      if (F8)
+        hidden_forward_f8<ACT>(tD + lane, sa[1] * sw[1],
+                               reinterpret_cast<const float*>(sm + P.bf) + kHidden, 1.f / sa[2],
+                               W + P.H2, W + P.S8, W + P.G2, row, hf, am[2]);
+      else
+        hidden_forward<ACT>(tD + lane, W + P.H2, W + P.G2, P.h3 ? W + P.H3 : nullptr, row, hf);
+      tc::fence_before_sync();
+      tc::fence_proxy_async();
+    }
+    if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
 
     // ---- third hidden layer (Sec. 4.4) -------------------------------------------
     if (P.h3) {
@@ -1159,11 +1164,13 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
         tc::mma_commit(bar);
       }
       wait_phase(bar, phase, bad);
-      tc::fence_after_sync();
-      hidden_forward<ACT>(tD + lane, W + P.H3, W + P.G3, nullptr, row, hf);
-      tc::fence_before_sync();
-      tc::fence_proxy_async();
-      tc::bar_sync(bar_id, kPipe);
+      if (!bad) {
+        tc::fence_after_sync();
+        hidden_forward<ACT>(tD + lane, W + P.H3, W + P.G3, nullptr, row, hf);
+        tc::fence_before_sync();
+        tc::fence_proxy_async();
+      }
+      if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
     }
 
     // ---- layer 3, loss, dZ3 ----------------------------------------------------
@@ -1178,51 +1185,53 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
       tc::mma_commit(bar);
     }
     wait_phase(bar, phase, bad);
-    tc::fence_after_sync();
-    {
-      // channels 8 hf .. 8 hf + 7
-      float zv[8];
-      tc::tmem_ld8(tD + lane + 8 * hf, zv);
-      tc::tmem_ld_wait();
-      if (F8) {
-        const float* b3 = reinterpret_cast<const float*>(sm + P.bf) + 2 * kHidden + 8 * hf;
+    if (!bad) {
+      tc::fence_after_sync();
+      {
+        // channels 8 hf .. 8 hf + 7
+        float zv[8];
+        tc::tmem_ld8(tD + lane + 8 * hf, zv);
+        tc::tmem_ld_wait();
+        if (F8) {
+          const float* b3 = reinterpret_cast<const float*>(sm + P.bf) + 2 * kHidden + 8 * hf;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) zv[c] = fmaf(zv[c], sa[2] * sw[2], b3[c]);
-      }
-      // dY from the target texel (loss mode) or the upstream gradient row (dout
-      // mode), without a branch per channel
-      const bool ident = M.out_act == NTC_OUT_IDENTITY;
-      const int live = valid ? C - 8 * hf : 0;  // channels of this half that count
-      float yc[8], dy[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        // sigmoid; the fast division is within 2 ulp
-        const float sg = __fdividef(1.f, 1.f + __expf(-zv[c]));
-        yc[c] = ident ? zv[c] : sg;
-      }
-      if (A.target) {
+          for (int c = 0; c < 8; ++c) zv[c] = fmaf(zv[c], sa[2] * sw[2], b3[c]);
+        }
+        // dY from the target texel (loss mode) or the upstream gradient row (dout
+        // mode), without a branch per channel
+        const bool ident = M.out_act == NTC_OUT_IDENTITY;
+        const int live = valid ? C - 8 * hf : 0;  // channels of this half that count
+        float yc[8], dy[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          const float t = (float)((tw[c >> 2] >> (8 * (c & 3))) & 0xFFu) * (1.f / 255.f);
-          const float e = c < live ? yc[c] - t : 0.f;
-          loss_acc = fmaf(e, e, loss_acc);
-          dy[c] = 2.f * e;
+          // sigmoid; the fast division is within 2 ulp
+          const float sg = __fdividef(1.f, 1.f + __expf(-zv[c]));
+          yc[c] = ident ? zv[c] : sg;
         }
-      } else {
+        if (A.target) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) dy[c] = c < live ? A.dout[i * C + 8 * hf + c] * dscale : 0.f;
-      }
-      float v[8];
+          for (int c = 0; c < 8; ++c) {
+            const float t = (float)((tw[c >> 2] >> (8 * (c & 3))) & 0xFFu) * (1.f / 255.f);
+            const float e = c < live ? yc[c] - t : 0.f;
+            loss_acc = fmaf(e, e, loss_acc);
+            dy[c] = 2.f * e;
+          }
+        } else {
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const float g = ident ? dy[c] : dy[c] * yc[c] * (1.f - yc[c]);
-        v[c] = c < live ? g : 0.f;
+          for (int c = 0; c < 8; ++c) dy[c] = c < live ? A.dout[i * C + 8 * hf + c] * dscale : 0.f;
+        }
+        float v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float g = ident ? dy[c] : dy[c] * yc[c] * (1.f - yc[c]);
+          v[c] = c < live ? g : 0.f;
+        }
+        put_chunk(W + P.DZ3, row, hf, v);
       }
-      put_chunk(W + P.DZ3, row, hf, v);
+      tc::fence_before_sync();
+      tc::fence_proxy_async();
     }
-    tc::fence_before_sync();
-    tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kPipe);
+    if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
 
     // ---- dHL = dZ3 W3; [dW3^T; db3] += [HL^T; 1] dZ3; then dZL over HL -------
     if (pw == 0 && tc::elect_one()) {
@@ -1232,11 +1241,13 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
       tc::mma_commit(bar);
     }
     wait_phase(bar, phase, bad);
-    tc::fence_after_sync();
-    hidden_backward<ACT, F8>(tD + lane, W + (P.h3 ? P.G3 : P.G2), W + P.HL, row, hf, sw[2]);
-    tc::fence_before_sync();
-    tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kPipe);
+    if (!bad) {
+      tc::fence_after_sync();
+      hidden_backward<ACT, F8>(tD + lane, W + (P.h3 ? P.G3 : P.G2), W + P.HL, row, hf, sw[2]);
+      tc::fence_before_sync();
+      tc::fence_proxy_async();
+    }
+    if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
 
     // ---- third layer: dH2 = dZh Wh; [dWh dbh] += dZh^T [H2 | 1]; dZ2 over H2 --
     if (P.h3) {
@@ -1247,11 +1258,13 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
         tc::mma_commit(bar);
       }
       wait_phase(bar, phase, bad);
-      tc::fence_after_sync();
-      hidden_backward<ACT, F8>(tD + lane, W + P.G2, W + P.H2, row, hf);
-      tc::fence_before_sync();
-      tc::fence_proxy_async();
-      tc::bar_sync(bar_id, kPipe);
+      if (!bad) {
+        tc::fence_after_sync();
+        hidden_backward<ACT, F8>(tD + lane, W + P.G2, W + P.H2, row, hf);
+        tc::fence_before_sync();
+        tc::fence_proxy_async();
+      }
+      if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
     }
 
     // ---- dH1 = dZ2 W2; [dW2 db2] += dZ2^T [H1 | 1]; then dZ1 over H1 ----------
@@ -1262,11 +1275,13 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
       tc::mma_commit(bar);
     }
     wait_phase(bar, phase, bad);
-    tc::fence_after_sync();
-    hidden_backward<ACT, F8>(tD + lane, W + P.G1, W + P.H1, row, hf, sw[1]);
-    tc::fence_before_sync();
-    tc::fence_proxy_async();
-    tc::bar_sync(bar_id, kPipe);
+    if (!bad) {
+      tc::fence_after_sync();
+      hidden_backward<ACT, F8>(tD + lane, W + P.G1, W + P.H1, row, hf, sw[1]);
+      tc::fence_before_sync();
+      tc::fence_proxy_async();
+    }
+    if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
 
     // ---- dX = dZ1 W1; [dW1 db1] += dZ1^T X ------------------------------------
     if (pw == 0 && tc::elect_one()) {
@@ -1323,7 +1338,7 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
       // then G0 per tap slot (weight 1; learned interpolation) or through
       // the bilinear taps, and G1 through the bilinear taps
       float* dxs = reinterpret_cast<float*>(W) + row * kDxStride;
-      for (int cb = 16 * hf; cb < P.dx_n; cb += 32) {
+      for (int cb = 16 * hf; !bad && cb < P.dx_n; cb += 32) {
         float v[16];
         tc::tmem_ld16(tD + lane + cb, v);
         tc::tmem_ld_wait();
@@ -1339,8 +1354,8 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
         // 4 (j % 4) .. +3 texel by texel, once per run of equal cells
         const int ln = tid & 31, wq = warp & 3;
         uint8_t* mbase = W + kRows * kDxStride * 4 + wq * 32 * kScatMeta;
-        put_meta(mbase + ln * kScatMeta);
-        tc::bar_sync(bar_id, kPipe);
+        if (!bad) put_meta(mbase + ln * kScatMeta);
+        if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
         const int k = ln >> 4, slot = ln >> 2, q = ln & 3;
         if (4 * q < (k ? M.c1 : M.c0)) {
           const int col = (k ? 8 * P.f0 : (LEARNED ? ((ln >> 2) & 3) * M.c0 : 0)) + 4 * q;
@@ -1354,7 +1369,8 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
           put_run(runs, open);
         }
       } else {
-        tc::bar_sync(bar_id, kPipe);  // both halves of the row are staged
+        // both halves of the row are staged
+        if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
         const float* dxs = reinterpret_cast<const float*>(W) + row * kDxStride;
         const int j = tb->level[m];
         const int wm = tb->wm[m], hm = tb->hm[m];
@@ -1387,7 +1403,7 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
       uint8_t* ws = W + (warp & 3) * kScatWarp;
       float* dxr = reinterpret_cast<float*>(ws) + ln * kScatDx;
       uint8_t* mr = ws + 32 * kScatDx * 4 + ln * kScatMeta;
-      {
+      if (!bad) {
         float v[16];
         tc::tmem_ld16(tD + lane + 16 * hf, v);
         tc::tmem_ld_wait();
@@ -1395,9 +1411,9 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
         for (int q = 0; q < 4; ++q)
           *reinterpret_cast<float4*>(dxr + 16 * hf + 4 * q) =
               make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        put_meta(mr);
       }
-      put_meta(mr);
-      tc::bar_sync(bar_id, kPipe);
+      if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
       {
         const int k = ln >> 4, slot = ln >> 2, q = ln & 3;
         const int col = (k ? 8 * P.f0 : 0) + 4 * q;
@@ -1418,6 +1434,7 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
     } else if (A.grids) {
       // dX slots: G0 at columns 0.., G1 at 8 * f0.. (f0 is 1 or 2); a half
       // scatters one grid
+      if (tc::bar_or(bar_id, kPipe, bad)) { bad = true; break; }
       float d[16];
       tc::tmem_ld16(tD + lane + (hf ? 8 * P.f0 : 0), d);
       tc::tmem_ld_wait();
