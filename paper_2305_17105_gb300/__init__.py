@@ -288,7 +288,8 @@ class Material:
         if w[1] is not None:
             wh, bh = w[1].data_ptr(), b[1].data_ptr()
         lv = []
-        for g0, g1 in zip(self.grids0, self.grids1):
+        for j in range(self.levels):
+            g0, g1 = self.grids0[j], self.grids1[j]
             s0, s1 = g0.shape, g1.shape
             lv += (s0[1], s0[0], s1[1], s1[0], g0.data_ptr(), g1.data_ptr())
         lv += (0,) * (6 * (MAX_LEVELS - self.levels))
