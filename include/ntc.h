@@ -288,8 +288,9 @@ size_t ntc_decode_host_workspace_bytes(int32_t channels, int32_t out_dtype, int6
 
 /* Launch shape of the tensor-core decode: warpgroup tile pipelines per CTA
  * (one CTA per SM, 128 TMEM columns per pipeline), 2, 3 or 4, or 5 for the
- * warp-specialised form (five compute warpgroups, four for layouts without a
- * kernel of their own, whose MMA chains other warps issue; FP16 and FP8); 0 restores the default (5).
+ * warp-specialised form (five compute warpgroups of 96 TMEM columns, four for
+ * layouts without a kernel of their own, whose MMA chains other warps issue;
+ * FP16 and FP8); 0 restores the default (5).
  * Process-wide; takes effect for later ntc_decode calls. */
 int ntc_set_decode_warpgroups(int32_t nwg);
 

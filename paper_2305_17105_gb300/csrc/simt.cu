@@ -362,7 +362,7 @@ __global__ void f8_scales_kernel(const uint32_t* amax, float* sa) {
 // one tile, hence small tiles spread over all SMs, with the rows' features
 // split over the warps (G0, G1, the encoding and target, the taps).  Tiles
 // of 128 texels, one per thread, ran a 4,096-texel step of a 256^2 x 8
-// material on 32 CTAs in 118 us (all launches of the step) against 36 now.
+// material on 32 CTAs in 118 us (all launches of the step) against 37 now.
 // ---------------------------------------------------------------------------
 constexpr int kBTile = 32;
 constexpr int kBThreads = 128;

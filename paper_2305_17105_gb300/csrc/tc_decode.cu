@@ -277,8 +277,9 @@ bool fast_layout_ok(const ntc_material& m) {
 
 // Launch shape: one CTA per SM with `nwg` warpgroup pipelines (2, 3 or 4),
 // each holding 128 of the SM's 512 TMEM columns, or (5, the default for 0)
-// the warp-specialised form: 4 compute warpgroups plus their MMA issuers
-// (FP16 and FP8).
+// the warp-specialised form: five compute warpgroups of 96 columns (four for
+// the layouts read from the plan) and warps that issue their MMAs (FP16 and
+// FP8).
 cudaError_t launch_decode_tc(const ntc_material& m, const float* uvl, int64_t n, void* out,
                              int out_dtype, int filter, uint64_t jkey, cudaStream_t s, int nwg) {
   if (n == 0) return cudaSuccess;

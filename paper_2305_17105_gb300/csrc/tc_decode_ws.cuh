@@ -35,7 +35,7 @@ namespace {
 // in flight hide part (issue slots half used, L1 three quarters).  96 columns
 // instead of 112 let a fifth pipeline in, and the issuers keep a chain's
 // steps 43 cycles apart (tc::elect_one): 2^24 random queries of a 4096^2 x 16
-// material 579 -> 517 us (1,450 GB/s of queries and outputs, 486 TFLOP/s), a
+// material 579 -> 518 us (1,450 GB/s of queries and outputs, 486 TFLOP/s), a
 // trilinear 3840 x 2160 frame 2,167 -> 1,768 us, in FP8 at 1080p 694 -> 594.
 // ---------------------------------------------------------------------------
 constexpr int kWsCompute = 4;  // many-material kernel

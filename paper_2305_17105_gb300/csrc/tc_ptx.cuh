@@ -43,17 +43,15 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;                // base offset 0, relative LBO mode, layout type 0 (no swizzle)
 }
 
-// One lane of a converged warp, the same one every time.  tcgen05.mma takes
-// its operands from uniform registers: inside `if (elect_one())`, with
-// warp-uniform operands, a chain with A in TMEM advances 43 cycles a step
-// (N = 64); issued under a divergent `lane == 0`, 95.
 // Programmatic dependent launch: wait until the kernel this one was launched
 // behind has completed and its writes are visible (at once when the launch was
 // an ordinary one).
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// The kernel launched behind this one may take its place on the chip.
-__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// One lane of a converged warp, the same one every time.  tcgen05.mma takes
+// its operands from uniform registers: inside `if (elect_one())`, with
+// warp-uniform operands, a chain with A in TMEM advances 43 cycles a step
+// (N = 64); issued under a divergent `lane == 0`, 95.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));

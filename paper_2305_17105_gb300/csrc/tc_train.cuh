@@ -10,7 +10,7 @@
 // step is bound by the latency of a tile's serial chain (issue slots a quarter
 // used).  With one thread a row and the MMAs issued by a divergent thread a
 // tile alone took 12.6 us against 8.9; a step of 2^18 texels of a 2048^2 x 12
-// material 176 -> 154 us, of eight crops on the paper's decoder 353 -> 259 us.
+// material 176 -> 150 us, of eight crops on the paper's decoder 353 -> 256 us.
 // Per tile, with every activation kept on chip:
 //   forward   X -> Z1 = X W1^T (+b1) -> H1 = act(Z1) -> Z2 (+b2) -> H2 -> Z3 (+b3)
 //             -> y = out(Z3), loss, dZ3 = 2 (y - t) out'(Z3); with a third
@@ -1633,9 +1633,14 @@ int pipelines_for(const ntc_material& m, int k_lay, int dx_lay) {
 int train_pipelines(const ntc_material& m) { return pipelines_for(m, 0, 0); }
 
 // Pipelines per CTA: the autotuner's choice (a.pipelines), else two (a third
-// would leave 80 registers a thread and take L1 from the gathers: 2^18 texels
-// of a 2048^2 x 12 material 102 us against 115 with three, as crops 80
-// against 81), or one for a call with no more tiles than SMs.
+// leaves 80 registers a thread and takes L1 from the gathers), or one for a
+// call with no more tiles than SMs.  A step with 1 / 2 / 3, us: 2^18 texels of
+// a 2048^2 x 12 material 183 / 150 / 160, ten materials of 2^16 texels each
+// 462 / 386 / 397; gradients of 2^18 texels in FP8 164 / 128 / 152, hardGELU
+// 175 / 130 / 130, learned G0 192 / 158 (two is the most that fits), but 7 + 5
+// channels 177 / 180 / 196 and crops of 16 + 16 channels 133 / 93 / 90; of
+// 1,000 texels 36 / 37 / 43, learned G0 43 / 51, FP8 47 / 46 / 61; of 24,000
+// 45 / 38 / 44.
 template <int ACT, bool LEARNED, bool BATCHED, bool F8>
 cudaError_t launch_n(const ntc_material& m, const BwdArgs& a, const TrainBatchDev* hb,
                      int64_t tiles, int k_lay, int dx_lay, cudaStream_t s) {
