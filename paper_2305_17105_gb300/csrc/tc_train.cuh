@@ -1211,7 +1211,9 @@ __global__ void __launch_bounds__(kPipe* NWG, 1) train_tc_kernel(const ntc_mater
         if (A.target) {
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
-            const float t = (float)((tw[c >> 2] >> (8 * (c & 3))) & 0xFFu) * (1.f / 255.f);
+            // (rounded by itself: contracted into the difference it moves dZ3 across
+            // FP16 roundings, and a cell's gradient with it)
+            const float t = __fmul_rn((float)((tw[c >> 2] >> (8 * (c & 3))) & 0xFFu), 1.f / 255.f);
             const float e = c < live ? yc[c] - t : 0.f;
             loss_acc = fmaf(e, e, loss_acc);
             dy[c] = 2.f * e;
