@@ -30,7 +30,7 @@ struct BwdArgs {
   int train;               // 1: loss mode (dout = 2 (y - t)), 0: dout given
   int grids;               // 0: skip grid gradients (frozen grids)
   int crops;               // training sampler: 256 x 256 crops of one mip (Sec. 5.1)
-  int pipelines;           // tensor-core step: pipelines per CTA (0: one or two, by the batch's tiles)
+  int pipelines;           // tensor-core step: pipelines per CTA (0: chosen by the batch's tiles)
   // Noise check folded into the tensor-core step (single material, bilinear
   // G0, grids of 4k <= 16 channels): with noisy_tag set, a CTA that finds it
   // current ({noise_seed, step}) gathers from the trainer's noisy copy

@@ -1,9 +1,9 @@
 // Tensor-core (tcgen05) fused forward + L2 loss + backward of the NTC
 // optimisation step (Sec. 4.2, 4.5, 5.1), FP16 operands, FP32 accumulation.
 //
-// One persistent CTA per SM runs NWG pipelines (two, one for calls with no
-// more tiles than SMs, up to three on request, as far as their tiles fit in
-// shared memory); a pipeline of 256 threads owns a stream of tiles of 128
+// One persistent CTA per SM runs NWG pipelines (one to three, chosen by the
+// call's tiles or on request, as far as their tiles fit in shared memory); a
+// pipeline of 256 threads owns a stream of tiles of 128
 // training texels (one row = one TMEM lane each).  Two threads share a row:
 // half 0 gathers G0, half 1 G1 and the encoding; in every epilogue each takes
 // one half of the columns, in the scatter one half of the warp's texels.  The
@@ -1635,19 +1635,23 @@ int pipelines_for(const ntc_material& m, int k_lay, int dx_lay) {
 int train_pipelines(const ntc_material& m) { return pipelines_for(m, 0, 0); }
 
 // Pipelines per CTA: the autotuner's choice (a.pipelines), else two (a third
-// leaves 80 registers a thread and takes L1 from the gathers), or one for a
-// call with no more tiles than SMs.  A step with 1 / 2 / 3, us: 2^18 texels of
-// a 2048^2 x 12 material 183 / 150 / 160, ten materials of 2^16 texels each
-// 462 / 386 / 397; gradients of 2^18 texels in FP8 164 / 128 / 152, hardGELU
-// 175 / 130 / 130, learned G0 192 / 158 (two is the most that fits), but 7 + 5
-// channels 177 / 180 / 196 and crops of 16 + 16 channels 133 / 93 / 90; of
-// 1,000 texels 36 / 37 / 43, learned G0 43 / 51, FP8 47 / 46 / 61; of 24,000
-// 45 / 38 / 44.
+// leaves 80 registers a thread and takes L1 from the gathers), one for a call
+// with no more tiles than SMs, or three where three take every tile at once and
+// two would not.  A step with 1 / 2 / 3, us: 2^18 texels of a 2048^2 x 12
+// material 183 / 150 / 160, ten materials of 2^16 texels each 462 / 386 / 397;
+// gradients of 2^18 texels in FP8 164 / 128 / 152, hardGELU 175 / 130 / 130,
+// learned G0 192 / 158 (two is the most that fits), but 7 + 5 channels 177 /
+// 180 / 196 and crops of 16 + 16 channels 133 / 93 / 90; of 1,000 texels 36 /
+// 37 / 43, learned G0 43 / 51, FP8 47 / 46 / 61; of 24,000 45 / 38 / 44.  Steps
+// of 45,000 texels (352 tiles) with two / three: 16 + 16 channels 54 / 47, 8 + 8
+// 43 / 38, 12 + 12 51 / 45, crops 47 / 41; of 38,000 (297) 40 / 45.
 template <int ACT, bool LEARNED, bool BATCHED, bool F8>
 cudaError_t launch_n(const ntc_material& m, const BwdArgs& a, const TrainBatchDev* hb,
                      int64_t tiles, int k_lay, int dx_lay, cudaStream_t s) {
   const int most = pipelines_for(m, k_lay, dx_lay);
-  const int want = a.pipelines > 0 ? a.pipelines : (tiles <= sm_count() ? 1 : 2);
+  const int64_t sms = sm_count();
+  const int at_once = tiles <= sms ? 1 : (tiles > 2 * sms && tiles <= 3 * sms ? 3 : 2);
+  const int want = a.pipelines > 0 ? a.pipelines : at_once;
   const int np = want < most ? want : most;
   switch (np) {
     case 3: return launch_t<ACT, LEARNED, 3, BATCHED, F8>(m, a, hb, tiles, k_lay, dx_lay, s);
