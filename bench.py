@@ -47,7 +47,7 @@ MAX_SM_MHZ = 2070.0
 # taken on (their hash), null otherwise.
 DECODE_SOURCES = ("tc_decode_ws.cuh", "tc_decode_common.cuh", "tc_decode_ws.cu", "tc_ptx.cuh",
                   "ntc_device.cuh")
-DECODE_TRAFFIC = ("6af1ee09e7d63671", 213.02e6 + 483.10e6)  # (sources sha256[:16], bytes per launch)
+DECODE_TRAFFIC = ("5267465a7b40727e", 213.33e6 + 482.42e6)  # (sources sha256[:16], bytes per launch)
 
 
 def decode_sources_sha():
